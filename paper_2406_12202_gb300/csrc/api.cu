@@ -363,12 +363,13 @@ static int render_passes(mcl_map* m, const float* d_poses, int N, const mcl_intr
                                            with_obs ? m->obs : nullptr),
                              "raygen")))
             return rc;
-        if (o->precision != MCL_PREC_FP32 &&
-            (rc = cuda_check(mlp_tc_ray_bias(m, m->gd, nr, nullptr, s), "per-ray bias")))
-            return rc;
+        if ((rc = cuda_check(mlp_tc_ray_bias(m, m->gd, nr, nullptr, s), "per-ray bias"))) return rc;
     }
-    auto mlp = [&](const float* z, int S, float4* dst, const FuseArgs* fa) -> cudaError_t {
-        if (o->precision == MCL_PREC_FP32) return mlp_fp32(m, m->rays, m->gd, z, S, nr, dst, s);
+    // (the FP32 form: the densities of a pass that importance samples are
+    // drawn from are those of the FMA chain)
+    auto mlp = [&](const float* z, int S, float4* dst, const FuseArgs* fa, bool first) -> cudaError_t {
+        if (o->precision == MCL_PREC_FP32)
+            return mlp_fp32(m, m->rays, z, S, nr, dst, s, nullptr, first && o->n_fine > 0);
         return mlp_tc(m, o->precision, m->rays, m->gd, z, S, nr, nullptr, dst, s, fa);
     };
     out->factor = f;
@@ -382,20 +383,20 @@ static int render_passes(mcl_map* m, const float* d_poses, int N, const mcl_intr
             fa2.S1 = o->n_fine > 0 ? o->n_coarse : 0;
             {
                 PhaseScope ph(m, MCL_PHASE_MLP_COARSE, s);
-                if ((rc = cuda_check(mlp(m->zc, o->n_coarse, m->out_c, o->n_fine > 0 ? &fa1 : &fa2),
+                if ((rc = cuda_check(mlp(m->zc, o->n_coarse, m->out_c, o->n_fine > 0 ? &fa1 : &fa2, true),
                                      "mlp (coarse, fused)")))
                     return rc;
             }
             if (o->n_fine > 0) {
                 PhaseScope ph(m, MCL_PHASE_MLP_FINE, s);
-                if ((rc = cuda_check(mlp(m->zf, o->n_fine, m->out_f, &fa2), "mlp (fine, fused)")))
+                if ((rc = cuda_check(mlp(m->zf, o->n_fine, m->out_f, &fa2, false), "mlp (fine, fused)")))
                     return rc;
             }
             return MCL_OK;
         }
         {
             PhaseScope ph(m, MCL_PHASE_MLP_COARSE, s);
-            if ((rc = cuda_check(mlp(m->zc, o->n_coarse, m->out_c, nullptr), "mlp (coarse)"))) return rc;
+            if ((rc = cuda_check(mlp(m->zc, o->n_coarse, m->out_c, nullptr, true), "mlp (coarse)"))) return rc;
         }
         if (o->n_fine > 0) {
             {
@@ -406,7 +407,7 @@ static int render_passes(mcl_map* m, const float* d_poses, int N, const mcl_intr
                     return rc;
             }
             PhaseScope ph(m, MCL_PHASE_MLP_FINE, s);
-            if ((rc = cuda_check(mlp(m->zf, o->n_fine, m->out_f, nullptr), "mlp (fine)"))) return rc;
+            if ((rc = cuda_check(mlp(m->zf, o->n_fine, m->out_f, nullptr, false), "mlp (fine)"))) return rc;
         }
         *out = Passes{m->zc, m->out_c, o->n_coarse, m->zf, m->out_f, o->n_fine, f, false};
         return MCL_OK;
@@ -434,20 +435,20 @@ static int render_passes(mcl_map* m, const float* d_poses, int N, const mcl_intr
         fa2.S1 = o->n_fine > 0 ? o->n_guided : 0;
         {
             PhaseScope ph(m, MCL_PHASE_MLP_COARSE, s);
-            if ((rc = cuda_check(mlp(m->zf, o->n_guided, m->out_c, o->n_fine > 0 ? &fa1 : &fa2),
+            if ((rc = cuda_check(mlp(m->zf, o->n_guided, m->out_c, o->n_fine > 0 ? &fa1 : &fa2, true),
                                  "mlp (guided, fused)")))
                 return rc;
         }
         if (o->n_fine > 0) {
             PhaseScope ph(m, MCL_PHASE_MLP_FINE, s);
-            if ((rc = cuda_check(mlp(m->zc, o->n_fine, m->out_f, &fa2), "mlp (fine, fused)")))
+            if ((rc = cuda_check(mlp(m->zc, o->n_fine, m->out_f, &fa2, false), "mlp (fine, fused)")))
                 return rc;
         }
         return MCL_OK;
     }
     {
         PhaseScope ph(m, MCL_PHASE_MLP_COARSE, s);
-        if ((rc = cuda_check(mlp(m->zf, o->n_guided, m->out_c, nullptr), "mlp (guided)"))) return rc;
+        if ((rc = cuda_check(mlp(m->zf, o->n_guided, m->out_c, nullptr, true), "mlp (guided)"))) return rc;
     }
     if (o->n_fine > 0) {
         {
@@ -458,7 +459,7 @@ static int render_passes(mcl_map* m, const float* d_poses, int N, const mcl_intr
                 return rc;
         }
         PhaseScope ph(m, MCL_PHASE_MLP_FINE, s);
-        if ((rc = cuda_check(mlp(m->zc, o->n_fine, m->out_f, nullptr), "mlp (fine)"))) return rc;
+        if ((rc = cuda_check(mlp(m->zc, o->n_fine, m->out_f, nullptr, false), "mlp (fine)"))) return rc;
     }
     *out = Passes{m->zf, m->out_c, o->n_guided, m->zc, m->out_f, o->n_fine, f, false};
     return MCL_OK;
@@ -516,9 +517,9 @@ extern "C" int mcl_query(mcl_map* m, const float* d_x, const float* d_dir, int n
     int rc;
     if ((rc = cuda_check(launch_query_setup(d_x, d_dir, n, m->rays, m->gd, m->zc, s), "query setup")))
         return rc;
-    if (precision == MCL_PREC_FP32)
-        return cuda_check(mlp_fp32(m, m->rays, m->gd, m->zc, 1, n, (float4*)d_out, s), "query mlp");
     if ((rc = cuda_check(mlp_tc_ray_bias(m, m->gd, n, nullptr, s), "query ray bias"))) return rc;
+    if (precision == MCL_PREC_FP32)
+        return cuda_check(mlp_fp32(m, m->rays, m->zc, 1, n, (float4*)d_out, s), "query mlp");
     return cuda_check(mlp_tc(m, precision, m->rays, m->gd, m->zc, 1, n, nullptr, (float4*)d_out, s),
                       "query mlp");
 }

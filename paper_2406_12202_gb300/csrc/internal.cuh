@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <functional>
 #include <vector>
 
 #include "../../include/mcl.h"
@@ -92,6 +93,7 @@ struct mcl_map {
     void* tc_blob = nullptr;
     size_t tc_bytes = 0;
     void* tc_aux = nullptr;
+    void* split = nullptr;          // FP32 form (filled by mlp_split_prepare)
     // workspace
     mcl::Ray* rays = nullptr;     // [max_rays]
     float* gd = nullptr;          // [max_rays, 32] gamma(d)
@@ -104,7 +106,7 @@ struct mcl_map {
     double* logw64 = nullptr;     // [max_particles]
     unsigned long long* cdf = nullptr;  // [max_particles] resampling CDF
     mcl::Status* status = nullptr;
-    // FP32-form activations (chunked)
+    // FP32 activations of the SIMT kernels (chunked)
     float* act0 = nullptr;
     float* act1 = nullptr;
     float* gxbuf = nullptr;
@@ -165,12 +167,21 @@ cudaError_t launch_weights(const float* e_ray, int N, int B, const mcl_opts& o, 
                            double* logw64, double* w, uint8_t* mask, float* S_dbg,
                            Status* status, cudaStream_t s);
 
-// mlp_fp32.cu: (sigma_raw, rgb) for rows r = ray*S + k of the pass.
-// rows_dev (optional): device-side row count (n_rays * S is the bound).
-cudaError_t mlp_fp32(mcl_map* m, const Ray* rays, const float* gd, const float* z, int S,
-                     int n_rays, float4* out, cudaStream_t s, const int* rows_dev = nullptr);
+// mlp_split.cu: the FP32 form, (sigma_raw, rgb) for rows r = ray*S + k of the
+// pass (the rays' colour-head bias from mlp_tc_ray_bias).  rows_dev
+// (optional): device-side row count (n_rays * S is the bound).
+// chain_density: the densities are those of the SIMT kernels' FMA chain.
+int mlp_split_prepare(mcl_map* m, const std::function<double(int, int, int)>& W,
+                      const float* const* bias, const float* w_out, const float* b_out);
+void mlp_split_free(mcl_map* m);
+cudaError_t mlp_fp32(mcl_map* m, const Ray* rays, const float* z, int S, int n_rays, float4* out,
+                     cudaStream_t s, const int* rows_dev = nullptr, bool chain_density = false);
 
-// mlp_fp32.cu building blocks reused by the map fitter (fit.cu): the FP32
+// mlp_fp32.cu: the same on the SIMT units; only_density: out.x alone.
+cudaError_t mlp_fp32_simt(mcl_map* m, const Ray* rays, const float* z, int S, int n_rays,
+                          float4* out, cudaStream_t s, const int* rows_dev, bool only_density);
+
+// mlp_fp32.cu, building blocks of the map fitter (fit.cu): the FP32
 // GEMM C = act([A1 | A2] W^T + b) (W [n_out][K1 + K2], n_out a multiple of
 // 128, K1 and K2 multiples of 16), gamma(x) of points (rays with z = 0), and
 // the density / colour heads (h [n,256] -> out.x; hid [n,256-stride] -> out.yzw).
@@ -206,6 +217,7 @@ bool mlp_tc_tuned(const mcl_map* m, int precision);
 int mlp_tc_hold_weights(mcl_map* m, int n_launches, unsigned long long wait_ns);
 cudaError_t mlp_tc_ray_bias(mcl_map* m, const float* gd, int n_rays, const int* n_rays_dev,
                             cudaStream_t s);
+const float* mlp_tc_ray_bias_buffer(const mcl_map* m);   // [max_rays][128], its result
 // Fused ray epilogue of a tensor-core MLP pass (tiles hold whole rays).
 //   mode 1 (first pass of the hierarchical sampler): Eq. 1 weights of each
 //          ray's S samples -> nf_out inverse-CDF samples into z_out [rays,

@@ -281,8 +281,8 @@ int enqueue_localize(mcl_map* m, int nq, float* P_user, int stride, const mcl_in
     fa2.obs = m->obs;
     fa2.e_ray = m->e_ray;
     auto mlp = [&](const float* z, int S, const int* rows_dev, float4* dst,
-                   const FuseArgs* fa) -> cudaError_t {
-        if (fp32) return mlp_fp32(m, m->rays, m->gd, z, S, max_rays_run, dst, s, rows_dev);
+                   const FuseArgs* fa, bool first) -> cudaError_t {
+        if (fp32) return mlp_fp32(m, m->rays, z, S, max_rays_run, dst, s, rows_dev, first && nf > 0);
         return mlp_tc(m, o.precision, m->rays, m->gd, z, S, max_rays_run, rows_dev, dst, s,
                       fused ? fa : nullptr);
     };
@@ -298,8 +298,8 @@ int enqueue_localize(mcl_map* m, int nq, float* P_user, int stride, const mcl_in
             L.plan, nq, Pc, stride, L.pix, K.fx, K.fy, K.cx, K.cy, np, o.near_z, o.far_z,
             prop ? 0 : o.jitter, o.seed, t, max_rays_run, m->rays, m->gd, m->zc, L.imgs, K.width,
             K.height, fused ? m->obs : nullptr);
-        if (!fp32 && (rc = cuda_check(mlp_tc_ray_bias(m, m->gd, max_rays_run, &L.plan->total_rays, s),
-                                      "loop ray bias")))
+        if ((rc = cuda_check(mlp_tc_ray_bias(m, m->gd, max_rays_run, &L.plan->total_rays, s),
+                             "loop ray bias")))
             return rc;
         if (prop) {
             if ((rc = cuda_check(launch_prop_infer(m, o.precision, m->rays, m->zc, np, max_rays_run,
@@ -310,7 +310,7 @@ int enqueue_localize(mcl_map* m, int nq, float* P_user, int stride, const mcl_in
                                  "loop proposal sampling")))
                 return rc;
         }
-        if ((rc = cuda_check(mlp(za, nc, &L.plan->rows_c, m->out_c, nf > 0 ? &fa1 : &fa2),
+        if ((rc = cuda_check(mlp(za, nc, &L.plan->rows_c, m->out_c, nf > 0 ? &fa1 : &fa2, true),
                              "loop mlp (coarse)")))
             return rc;
         if (nf > 0) {
@@ -319,7 +319,7 @@ int enqueue_localize(mcl_map* m, int nq, float* P_user, int stride, const mcl_in
                                                        za, nc, m->out_c, nf, zb, s),
                                  "loop importance sampling")))
                 return rc;
-            if ((rc = cuda_check(mlp(zb, nf, &L.plan->rows_f, m->out_f, &fa2), "loop mlp (fine)")))
+            if ((rc = cuda_check(mlp(zb, nf, &L.plan->rows_f, m->out_f, &fa2, false), "loop mlp (fine)")))
                 return rc;
         }
         if (!fused) {

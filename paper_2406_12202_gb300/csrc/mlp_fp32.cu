@@ -1,7 +1,9 @@
-// mlp_fp32.cu -- the plain FP32 form of the NeRF MLP: positional encoding,
-// one SIMT FP32 GEMM launch per layer with bias and ReLU, and two row-wise
-// head kernels.  Activations live in HBM (chunks of rows), so this form is
-// also the unfused comparison point for the tensor-core path.
+// mlp_fp32.cu -- the FP32 NeRF MLP on the SIMT units: positional encoding, one
+// FP32 GEMM launch per layer with bias and ReLU, and two row-wise head
+// kernels, activations in HBM (chunks of rows).  The map fitter (fit.cu)
+// builds on these kernels; maps with sparse weights run on them, and the
+// densities that importance samples are drawn from (see mlp_split.cu, which
+// holds the rest of the FP32 form).
 #include <math.h>
 
 #include "internal.cuh"
@@ -273,8 +275,9 @@ static cudaError_t gemm(const float* A1, int lda1, int K1, const float* A2, int 
     return cudaGetLastError();
 }
 
-cudaError_t mlp_fp32(mcl_map* m, const Ray* rays, const float* gd, const float* z, int S,
-                     int n_rays, float4* out, cudaStream_t s, const int* rows_dev) {
+cudaError_t mlp_fp32_simt(mcl_map* m, const Ray* rays, const float* z, int S, int n_rays,
+                          float4* out, cudaStream_t s, const int* rows_dev, bool only_density) {
+    const float* gd = m->gd;
     const long rows = (long)n_rays * S;
     cudaError_t e = cudaSuccess;
     for (long r0 = 0; r0 < rows; r0 += m->chunk_rows) {
@@ -303,6 +306,10 @@ cudaError_t mlp_fp32(mcl_map* m, const Ray* rays, const float* gd, const float* 
         note_launch();
         k_sigma_head<<<(n * 16 + 255) / 256, 256, 0, s>>>(a, kWidth, m->L[8].W, m->L[8].b, n,
                                                           rows_dev, r0, out + r0);
+        if (only_density) {
+            if ((e = cudaGetLastError())) return e;
+            continue;
+        }
         if ((e = gemm(a, kWidth, kWidth, nullptr, 0, 0, 0, 1, m->L[9], b, kWidth, n, false,
                       rows_dev, r0, s)))
             return e;

@@ -2454,11 +2454,13 @@ int mlp_tc_prepare(mcl_map* m, const float* blob) {
         st->max_pairs = std::min(st->max_pairs, st->n_sm / 2);
         if (st->max_pairs < 1) return fail(MCL_ERR_UNSUPPORTED, "no CTA pair fits on an SM pair");
     }
+    if ((rc = mlp_split_prepare(m, weight, bp, Wp[11], bp[11]))) return rc;
     st->bf16.ready = st->fp8.ready = st->bf16_split.ready = true;
     return MCL_OK;
 }
 
 void mlp_tc_free(mcl_map* m) {
+    mlp_split_free(m);
     TcState* st = (TcState*)m->tc_aux;
     if (!st) return;
     if (st->bf16.wblocks) cudaFree(st->bf16.wblocks);
@@ -2488,6 +2490,8 @@ cudaError_t mlp_tc_ray_bias(mcl_map* m, const float* gd, int n_rays, const int* 
                                                            st->bprime, st->ray_bias);
     return cudaGetLastError();
 }
+
+const float* mlp_tc_ray_bias_buffer(const mcl_map* m) { return ((const TcState*)m->tc_aux)->ray_bias; }
 
 static cudaError_t mlp_tc_variant(mcl_map* m, int precision, int variant, const Ray* rays,
                                   const float* z, int S, int n_rays, const int* rows_dev,
