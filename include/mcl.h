@@ -413,7 +413,7 @@ int mcl_get_map_weights(mcl_map* map, float* host_out, size_t n);
  *   3 FP8 8 lockstep    4 FP8 4 staggered   5 FP8 8 staggered
  *   6 BF16 4 split      7 BF16 4 pipelined (one tile per CTA)
  *   8 BF16 4 lockstep, CTA pair   9 FP8 4 lockstep, CTA pair
- *  10 FP8 4 staggered, CTA pair   11 BF16 4 staggered   12 BF16 8 staggered
+ *  10 FP8 8 staggered, CTA pair   11 BF16 4 staggered   12 BF16 8 staggered
  *  13 BF16 4 staggered, CTA pair
  * Lockstep: each streamed weight block serves both tiles of a pair at once;
  * staggered: the second tile runs each part of a layer (the blocks the
@@ -427,7 +427,7 @@ int mcl_get_map_weights(mcl_map* map, float* host_out, size_t n);
  * at a time as the epilogue writes them; CTA pair: clusters of two CTAs on
  * the two SMs of a TPC issue 256-row MMAs (tcgen05 cta_group::2), each CTA
  * streaming half of every weight block.  All variants of a precision give
- * bit-identical results.  Untuned defaults: 12 (BF16) and 5 (FP8). */
+ * bit-identical results.  Untuned defaults: 13 (BF16) and 5 (FP8). */
 #define MCL_MLP_VARIANTS 14
 
 /* Autotuner: time every variant of `precision` (MCL_PREC_BF16 or _FP8) on

@@ -620,7 +620,7 @@ MLP_VARIANT_TABLE = {0: ("bf16", 4, "lockstep"), 1: ("bf16", 8, "lockstep"),
                      4: ("fp8", 4, "staggered"), 5: ("fp8", 8, "staggered"),
                      6: ("bf16", 4, "split"), 7: ("bf16", 4, "pipelined"),
                      8: ("bf16", 4, "lockstep pair"), 9: ("fp8", 4, "lockstep pair"),
-                     10: ("fp8", 4, "staggered pair"), 11: ("bf16", 4, "staggered"),
+                     10: ("fp8", 8, "staggered pair"), 11: ("bf16", 4, "staggered"),
                      12: ("bf16", 8, "staggered"), 13: ("bf16", 4, "staggered pair")}
 
 # Weights of the learned proposal (gamma(x) with 6 frequencies -> 4 x 64 ReLU

@@ -215,9 +215,23 @@ int mlp_tc_autotune(mcl_map* m, int precision, long long rows, int* chosen, floa
                     cudaStream_t s);
 bool mlp_tc_tuned(const mcl_map* m, int precision);
 int mlp_tc_hold_weights(mcl_map* m, int n_launches, unsigned long long wait_ns);
+// points: the rays are point queries (one sample each) in `precision`.
 cudaError_t mlp_tc_ray_bias(mcl_map* m, const float* gd, int n_rays, const int* n_rays_dev,
-                            cudaStream_t s);
-const float* mlp_tc_ray_bias_buffer(const mcl_map* m);   // [max_rays][128], its result
+                            cudaStream_t s, bool points = false, int precision = MCL_PREC_FP32);
+// Its result: the 128 colour-head biases of a ray as 16-byte groups q (values
+// 4 q .. 4 q + 3) at [step q] of ray_bias_at.  Rays of many samples: one after
+// the other (step 1), a warp's rows share a ray and its lines.  Point queries:
+// 32 rays interleaved (step 32), so that the 32 rows of a warp, a ray each,
+// read whole lines (100,003 points in BF16: 238 -> 194 us; 262,144 in FP32:
+// 898 -> 782 us; interleaved, the rays of a full update would cost FP8 0.8 %).
+struct RayBias {
+    const float* buf;
+    int step;
+};
+RayBias mlp_tc_ray_bias_result(const mcl_map* m);
+__device__ __forceinline__ const float4* ray_bias_at(const RayBias& b, long long ray) {
+    return reinterpret_cast<const float4*>(b.buf) + (b.step == 1 ? ray * 32 : (ray >> 5) * 1024 + (ray & 31));
+}
 // Fused ray epilogue of a tensor-core MLP pass (tiles hold whole rays).
 //   mode 1 (first pass of the hierarchical sampler): Eq. 1 weights of each
 //          ray's S samples -> nf_out inverse-CDF samples into z_out [rays,

@@ -99,7 +99,7 @@ struct SplitParams {
     int S;
     long long M;                 // rows of the pass (upper bound with M_dev)
     const int* M_dev;            // optional: rows in device memory
-    const float* ray_bias;       // [n_rays][128]
+    RayBias ray_bias;
     float4* out;
     int* abort_flag;
     int* status_code;
@@ -512,10 +512,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             const long long row = ((long long)u * 2 + rank) * 128 + r;
             const bool valid = row < M;
             const long long ray = !valid ? 0 : M <= 0xffffffffll ? (long long)((uint32_t)row / (uint32_t)p.S) : row / p.S;
-            const float4* rb4 = reinterpret_cast<const float4*>(p.ray_bias + ray * 128 + j * 64);
+            const float4* rb4 = ray_bias_at(p.ray_bias, ray) + j * 16 * p.ray_bias.step;
 #pragma unroll
             for (int q = 0; q < 16; ++q) {
-                const float4 b = __ldg(rb4 + q);
+                const float4 b = __ldg(rb4 + q * p.ray_bias.step);
                 s[2 * q] = make_float2(b.x, b.y);
                 s[2 * q + 1] = make_float2(b.z, b.w);
             }
@@ -724,7 +724,7 @@ cudaError_t mlp_fp32(mcl_map* m, const Ray* rays, const float* z, int S, int n_r
     p.S = S;
     p.M = (long long)n_rays * S;
     p.M_dev = rows_dev;
-    p.ray_bias = mlp_tc_ray_bias_buffer(m);
+    p.ray_bias = mlp_tc_ray_bias_result(m);
     p.out = out;
     p.abort_flag = st->abort_flag;
     p.status_code = &m->status->code;

@@ -92,7 +92,7 @@ __host__ __device__ constexpr int layer_chunks(bool f8, int l) {
     return (l == 0 ? 2 : l == 5 ? 10 : 8) >> (f8 ? 1 : 0);
 }
 
-struct EpiConsts {
+struct __align__(16) EpiConsts {   // (16-byte constant loads)
     uint32_t bias2[8][128];   // BF16: trunk biases as BF16 pairs
     float beta[8][256];       // FP8: epilogue offset per column
     float alpha_last[128];    // FP8: dequantisation of the RGB hidden layer
@@ -112,7 +112,7 @@ struct Params {
     float alpha_sigma;      // FP8: dequantisation of the density head
     float s_gx;             // FP8: scale of gamma(x)
     float b_sigma;
-    const float* ray_bias;  // [n_rays][128]
+    RayBias ray_bias;       // per-ray colour-head bias
     float b_out0, b_out1, b_out2;
     float4* out;
     int* abort_flag;        // per-launch: set on a timed-out wait
@@ -199,11 +199,15 @@ __device__ __forceinline__ void epi_chunk_store(const uint32_t (&v)[32], const u
     const uint32_t one2 = 0x3F803F80u;  // (1.0, 1.0) in BF16
     uint32_t pk[16];
 #pragma unroll
-    for (int i = 0; i < 16; ++i) {
-        const uint32_t a = pack_bf16x2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));
-        uint32_t h;
-        asm("fma.rn.relu.bf16x2 %0, %1, %2, %3;" : "=r"(h) : "r"(a), "r"(one2), "r"(bias[i]));
-        pk[i] = h;
+    for (int q = 0; q < 4; ++q) {
+        const uint4 b4 = reinterpret_cast<const uint4*>(bias)[q];
+        const uint32_t b[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int i = 4 * q + e;
+            const uint32_t a = pack_bf16x2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));
+            asm("fma.rn.relu.bf16x2 %0, %1, %2, %3;" : "=r"(pk[i]) : "r"(a), "r"(one2), "r"(b[e]));
+        }
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q)
@@ -224,7 +228,7 @@ __device__ __forceinline__ void epi_chunk_store_f8(const uint32_t (&v)[32], floa
     for (int q = 0; q < 8; ++q) {
         float4 b;
         if constexpr (kGlobal) b = __ldg(reinterpret_cast<const float4*>(beta) + q);
-        else b = make_float4(beta[4 * q], beta[4 * q + 1], beta[4 * q + 2], beta[4 * q + 3]);
+        else b = reinterpret_cast<const float4*>(beta)[q];
         pk[q] = pack_e4m3x4_relu(fmaf(__uint_as_float(v[4 * q + 0]), alpha, b.x),
                                  fmaf(__uint_as_float(v[4 * q + 1]), alpha, b.y),
                                  fmaf(__uint_as_float(v[4 * q + 2]), alpha, b.z),
@@ -236,14 +240,16 @@ __device__ __forceinline__ void epi_chunk_store_f8(const uint32_t (&v)[32], floa
 
 // One 32-column group of the last layer: h = relu(acc (* alpha) + b_ray),
 // then the 128 -> 3 output layer as running dot products (wo [3][128] and
-// al [128]: the parameter block; rb4: the ray's bias in global memory).
-template <bool F8>
+// al [128]: the parameter block; rb4, STEP: the ray's bias in global memory,
+// see RayBias; a constant, since the 8-warp kernels have no register left for
+// it and two copies of the code cost them 2 to 3 %).
+template <bool F8, int STEP = 1>
 __device__ __forceinline__ void rgb_group(const uint32_t (&v)[32], const float4* rb4,
                                           const float* wo, const float* al, int c32,
                                           float& o0, float& o1, float& o2) {
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-        const float4 b = __ldg(rb4 + c32 * 8 + q);
+        const float4 b = __ldg(rb4 + (c32 * 8 + q) * STEP);
         const int c = c32 * 32 + 4 * q;
         float a0 = __uint_as_float(v[4 * q + 0]), a1 = __uint_as_float(v[4 * q + 1]);
         float a2 = __uint_as_float(v[4 * q + 2]), a3 = __uint_as_float(v[4 * q + 3]);
@@ -652,7 +658,7 @@ __device__ __forceinline__ void signal_ready(uint32_t bar, int lane) {
     tc_fence_before();
     if constexpr (PAIR) {
         __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(bar);
+        if (lane == 0) mbar_arrive_peer(bar);
     } else {
         mbar_arrive(bar);
     }
@@ -667,7 +673,7 @@ __device__ __forceinline__ void signal_ready(uint32_t bar, int lane) {
 // addresses of the even CTA's barriers.  FUSE (0, 1, 2): the fused ray
 // epilogue of the pass (Params::fuse); instantiations without it carry no
 // code or registers for it.
-template <bool F8, int EPIW, bool PAIR, int FUSE = 0>
+template <bool F8, int EPIW, bool PAIR, int FUSE = 0, bool POINTS = false>
 __device__ __forceinline__ void epilogue_warps(const Params& p, int warp, int warp0, int lane, uint32_t tmem,
                                                uint32_t s_act, uint32_t s_gx, uint32_t bar_ready0,
                                                uint32_t bar_ready1, uint32_t bar_acc0,
@@ -773,8 +779,7 @@ __device__ __forceinline__ void epilogue_warps(const Params& p, int warp, int wa
         const float zrow = nz, dnrow = ndn;
         float4 res = make_float4(0.f, 0.f, 0.f, 0.f);
         for (int l = 0; l < kLayers && ok; ++l) {
-            const bool got = PAIR ? mbar_wait_cluster<true>(bar_acc, acc_ph, abort_flag)
-                                  : mbar_wait_sleep(bar_acc, acc_ph, abort_flag, p.wait_ns);
+            const bool got = mbar_wait_sleep(bar_acc, acc_ph, abort_flag, p.wait_ns);
             if (!got) {
                 if constexpr (FUSE != 0) {
                     record_abort(p);
@@ -846,7 +851,8 @@ __device__ __forceinline__ void epilogue_warps(const Params& p, int warp, int wa
                     // (column 128) read out of TMEM in two bursts, so that
                     // the accumulator is soon free for the next unit's
                     // first layer
-                    const float4* rb4 = reinterpret_cast<const float4*>(p.ray_bias + ray * 128);
+                    const float4* rb4 = ray_bias_at(p.ray_bias, ray);
+                    constexpr int kStep = POINTS ? 32 : 1;
                     const float* wo = &p.ec.w_out[0][0];
                     float o0 = 0.f, o1 = 0.f, o2 = 0.f;
                     uint32_t va[32], vb[32];
@@ -872,15 +878,15 @@ __device__ __forceinline__ void epilogue_warps(const Params& p, int warp, int wa
                         if (p.obs && quad < 128 / p.S && ray0 + quad < n_rays) ob = p.obs[ray0 + quad];
                     }
                     tmem_ld_wait();
-                    rgb_group<F8>(va, rb4, wo, p.ec.alpha_last, 0, o0, o1, o2);
-                    rgb_group<F8>(vb, rb4, wo, p.ec.alpha_last, 1, o0, o1, o2);
+                    rgb_group<F8, kStep>(va, rb4, wo, p.ec.alpha_last, 0, o0, o1, o2);
+                    rgb_group<F8, kStep>(vb, rb4, wo, p.ec.alpha_last, 1, o0, o1, o2);
                     tmem_ld32(t_row + 64, va);
                     tmem_ld32(t_row + 96, vb);
                     tmem_ld1(t_row + 128, vs);
                     tmem_ld_wait();
                     if (has_next) signal_ready<PAIR>(bar_ready, lane);
-                    rgb_group<F8>(va, rb4, wo, p.ec.alpha_last, 2, o0, o1, o2);
-                    rgb_group<F8>(vb, rb4, wo, p.ec.alpha_last, 3, o0, o1, o2);
+                    rgb_group<F8, kStep>(va, rb4, wo, p.ec.alpha_last, 2, o0, o1, o2);
+                    rgb_group<F8, kStep>(vb, rb4, wo, p.ec.alpha_last, 3, o0, o1, o2);
                     float sigma = __uint_as_float(vs);
                     if constexpr (F8) sigma *= p.alpha_sigma;
                     res.x = sigma + p.b_sigma;
@@ -926,7 +932,7 @@ __device__ __forceinline__ void epilogue_warps(const Params& p, int warp, int wa
     if (!ok) record_abort(p);
 }
 
-template <bool F8, int EPIW, bool STAG, int FUSE = 0>
+template <bool F8, int EPIW, bool STAG, int FUSE = 0, bool POINTS = false>
 __global__ void __launch_bounds__(Variant<F8, EPIW, STAG>::kThreads, 1)
     k_mlp_tc(const __grid_constant__ Params p) {
     using Fm = Form<F8>;
@@ -1255,7 +1261,7 @@ __global__ void __launch_bounds__(Variant<F8, EPIW, STAG>::kThreads, 1)
         }
         if (!ok && lane == 0) record_abort(p);
     } else {
-        epilogue_warps<F8, EPIW, false, FUSE>(p, warp, 3, lane, tmem, s_act, s_gx,
+        epilogue_warps<F8, EPIW, false, FUSE, POINTS>(p, warp, 3, lane, tmem, s_act, s_gx,
                                         smem_u32(&bars.a_ready[0]), smem_u32(&bars.a_ready[1]),
                                         smem_u32(&bars.acc_full[0]), smem_u32(&bars.acc_full[1]),
                                         M, blockIdx.x, gridDim.x, n_pairs, 256, 0, smem,
@@ -1280,10 +1286,18 @@ __global__ void __launch_bounds__(Variant<F8, EPIW, STAG>::kThreads, 1)
 // The even CTA's warp 1 issues all MMAs, released by its gate warp once its
 // own copy of a block has landed (full[]) and the odd CTA's warp 1 has
 // relayed that the odd CTA's copy has (the even CTA's pfull[]); the
-// epilogue warps (3 .. 10) of both CTAs signal
+// epilogue warps (from warp 3 on) of both CTAs signal
 // the even CTA's a_ready[] barriers; the MMA commits arrive on the barriers
 // of both CTAs (multicast).  Same arithmetic per row as the single-CTA
-// kernel.
+// kernel.  Waits and arrivals are at CTA scope: what crosses the pair is the
+// tensor core's to order (proxy fence, commit), and at cluster scope every
+// acquire dropped the L1 and every release waited for all earlier stores
+// (2.46 M rows: staggered BF16 2.79 -> 2.02 ms, FP8 2.09 -> 1.70, with 8
+// epilogue warps per tile 1.52; BF16 with 8 warps 2.10).  What bounds the
+// BF16 pair now is the weight ring: a stage is free again only after tile 1's
+// MMAs, and its refill (commit, L2, relay, about 2,000 cycles) is due within
+// the 1,800 of the other tile's turn; parts of 1 to 4 blocks (2.09 to 2.25
+// ms) and waiting for runs of 2 to 8 blocks (2.04 to 2.50) are slower.
 template <bool F8>
 struct PairForm {
     static constexpr int kStages = 2 * Form<F8>::kStages;     // half-blocks
@@ -1293,7 +1307,8 @@ struct PairForm {
 };
 static_assert(PairForm<false>::kSmemBytes <= 232448 && PairForm<true>::kSmemBytes <= 232448, "smem");
 constexpr int kPairMaxStages = 16;
-constexpr int kPairThreads = 96 + 2 * 128;
+template <int EPIW>
+constexpr int kPairThreads = 96 + 2 * 32 * EPIW;
 
 struct __align__(8) PairBars {
     uint64_t full[kPairMaxStages];
@@ -1305,8 +1320,8 @@ struct __align__(8) PairBars {
     uint32_t tmem_base;
 };
 
-template <bool F8, bool STAG>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
+template <bool F8, int EPIW, bool STAG, bool POINTS = false>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads<EPIW>, 1)
     k_mlp_tc2(const __grid_constant__ Params p) {
     using Fm = Form<F8>;
     using Pf = PairForm<F8>;
@@ -1334,7 +1349,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
         }
         for (int s = 0; s < 2; ++s) {
             mbar_init(smem_u32(&bars.acc_full[s]), 1);
-            mbar_init(smem_u32(&bars.a_ready[s]), 8);   // 4 epilogue warps x 2 CTAs
+            mbar_init(smem_u32(&bars.a_ready[s]), 2 * EPIW);
         }
         mbar_init(smem_u32(&bars.drain), 1);
         fence_mbar_init();
@@ -1356,7 +1371,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
             for (long long u = u0; u < n_units && ok; u += du) {
                 for (int b = 0; b < Fm::kBlocks; ++b, ++g) {
                     const uint32_t st = g % kStages, ph = (g / kStages) & 1u;
-                    if (!mbar_wait_cluster<false>(smem_u32(&bars.empty[st]), ph ^ 1u, abort_flag)) {
+                    if (!mbar_wait(smem_u32(&bars.empty[st]), ph ^ 1u, abort_flag)) {
                         ok = false;
                         break;
                     }
@@ -1386,7 +1401,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
                         ok = false;
                         break;
                     }
-                    mbar_arrive_cluster(mapa_shared(smem_u32(&bars.pfull[st]), 0));
+                    mbar_arrive_peer(mapa_shared(smem_u32(&bars.pfull[st]), 0));
                 }
             if (!ok) record_abort(p);
         }
@@ -1509,7 +1524,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
             uint32_t rdy_ph = 0;   // bit s: phase parity of a_ready[s]
             bool ok = true;
             auto wait_ready = [&](int s) -> bool {
-                const bool r = mbar_wait_cluster<false>(smem_u32(&bars.a_ready[s]), (rdy_ph >> s) & 1u, abort_flag);
+                const bool r = mbar_wait(smem_u32(&bars.a_ready[s]), (rdy_ph >> s) & 1u, abort_flag);
                 rdy_ph ^= 1u << s;
                 return r;
             };
@@ -1517,7 +1532,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
             auto wait_block = [&](uint32_t gi) -> bool {
                 const uint32_t st = gi % kStages, ph = (gi / kStages) & 1u;
                 const bool r = mbar_wait(smem_u32(&bars.full[st]), ph, abort_flag);
-                const bool r2 = r && mbar_wait_cluster<false>(smem_u32(&bars.pfull[st]), ph, abort_flag);
+                const bool r2 = r && mbar_wait(smem_u32(&bars.pfull[st]), ph, abort_flag);
                 return r2;
             };
             auto release = [&](bool good) -> bool {
@@ -1538,14 +1553,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
                                 // failure, which stops the MMA warp)
                                 bool good = true;
                                 if (c == 0) good = wait_ready(0);
-                                good = good && wait_block(g + c);
                                 const int rem = c0 + np - c;
+                                good = good && wait_block(g + c);
                                 bool landed = lane == 0;
                                 if (lane > 0 && lane < rem) {
                                     const uint32_t gi = g + c + lane;
                                     const uint32_t st = gi % kStages, ph = (gi / kStages) & 1u;
                                     landed = mbar_try_wait(smem_u32(&bars.full[st]), ph) &&
-                                             mbar_try_wait_cluster(smem_u32(&bars.pfull[st]), ph);
+                                             mbar_try_wait(smem_u32(&bars.pfull[st]), ph);
                                 }
                                 const uint32_t m = __ballot_sync(0xffffffffu, landed);
                                 const int k = good ? __ffs(~m) - 1 : 0;
@@ -1574,7 +1589,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
     } else {
         const uint32_t rdy0 = mapa_shared(smem_u32(&bars.a_ready[0]), 0);
         const uint32_t rdy1 = mapa_shared(smem_u32(&bars.a_ready[1]), 0);
-        epilogue_warps<F8, 4, true>(p, warp, 3, lane, tmem, s_act, s_gx, rdy0, rdy1,
+        epilogue_warps<F8, EPIW, true, 0, POINTS>(p, warp, 3, lane, tmem, s_act, s_gx, rdy0, rdy1,
                                     smem_u32(&bars.acc_full[0]), smem_u32(&bars.acc_full[1]), M, u0, du,
                                     n_units, 512, (long long)rank * 256, smem);
     }
@@ -1776,7 +1791,7 @@ __global__ void __launch_bounds__(kSplitThreads, 1) k_mlp_tc_split(const __grid_
                 mbar_arrive(r_hi);
             }
             float o0 = 0.f, o1 = 0.f, o2 = 0.f;
-            const float4* rb4 = reinterpret_cast<const float4*>(p.ray_bias + ray * 128);
+            const float4* rb4 = ray_bias_at(p.ray_bias, ray);
             const float* wo = &p.ec.w_out[0][0];
             for (int l = 0; l < kLayers && ok; ++l) {
                 for (int h = 0; h < 2 && ok; ++h) {
@@ -2044,7 +2059,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1) k_mlp_tc_pipe(const __grid_co
                         mbar_arrive(smem_u32(&bars.q_ready[q]));
                     }
                 } else {
-                    const float4* rb4 = reinterpret_cast<const float4*>(p.ray_bias + ray * 128);
+                    const float4* rb4 = ray_bias_at(p.ray_bias, ray);
                     const float* wo = &p.ec.w_out[0][0];
                     float o0 = 0.f, o1 = 0.f, o2 = 0.f;
                     uint32_t va[32], vb[32];
@@ -2083,20 +2098,51 @@ __global__ void __launch_bounds__(kPipeThreads, 1) k_mlp_tc_pipe(const __grid_co
     }
 }
 
-// Per-ray bias of the RGB hidden layer: b'_ray = b' + W_rgb_hidden[:, 256:283] gamma(d).
-__global__ void k_ray_bias(const float* __restrict__ gd, int n_rays, const int* __restrict__ n_dev,
-                           const float* __restrict__ Wd, const float* __restrict__ bprime,
-                           float* __restrict__ out) {
-    const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
+// Per-ray bias of the RGB hidden layer: b'_ray = b' + W_rgb_hidden[:, 256:283]
+// gamma(d), in the layout of RayBias.  One after the other: a warp per ray, a
+// lane takes four outputs.  Interleaved: a block of 8 warps takes 32 rays, a
+// lane a ray, a warp four outputs of each at a time (the weights are then
+// broadcast loads).  Both store 512 bytes per warp, which is what bounds it.
+template <bool POINTS>
+__global__ void __launch_bounds__(256) k_ray_bias(const float* __restrict__ gd, int n_rays,
+                                                  const int* __restrict__ n_dev,
+                                                  const float* __restrict__ Wd,
+                                                  const float* __restrict__ bprime,
+                                                  float4* __restrict__ out) {
     const int n = n_dev ? min(n_rays, *n_dev) : n_rays;
-    if (t >= (long)n * 128) return;
-    const long ray = t >> 7;
-    const int o = (int)(t & 127);
-    const float* g = gd + ray * kGdPad;
-    float s = bprime[o];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const float4* W4 = reinterpret_cast<const float4*>(Wd);   // [27][128]
+    const float4* b4 = reinterpret_cast<const float4*>(bprime);
+    auto add = [&](float4& s, const float4& w, float x) {
+        s.x = fmaf(w.x, x, s.x);
+        s.y = fmaf(w.y, x, s.y);
+        s.z = fmaf(w.z, x, s.z);
+        s.w = fmaf(w.w, x, s.w);
+    };
+    if constexpr (POINTS) {
+        __shared__ float g[32][kGdPad + 1];
+        const int r0 = blockIdx.x * 32;
+        if (r0 >= n) return;
+        for (int t = threadIdx.x; t < 32 * kGdPad; t += 256) {
+            const int ray = r0 + t / kGdPad;
+            g[t / kGdPad][t % kGdPad] = ray < n ? gd[(size_t)ray * kGdPad + t % kGdPad] : 0.f;
+        }
+        __syncthreads();
+        for (int q = warp; q < 32; q += 8) {
+            float4 s = b4[q];
 #pragma unroll
-    for (int i = 0; i < kGd; ++i) s = fmaf(Wd[i * 128 + o], g[i], s);   // Wd: [27][128]
-    out[t] = s;
+            for (int i = 0; i < kGd; ++i) add(s, __ldg(W4 + i * 32 + q), g[lane][i]);
+            if (r0 + lane < n) out[(size_t)blockIdx.x * 1024 + q * 32 + lane] = s;
+        }
+    } else {
+        const long ray = (long)blockIdx.x * 8 + warp;
+        if (ray >= n) return;
+        const float x = gd[ray * kGdPad + lane];
+        float4 s = b4[lane];
+#pragma unroll
+        for (int i = 0; i < kGd; ++i) add(s, __ldg(W4 + i * 32 + lane), __shfl_sync(0xffffffffu, x, i));
+        out[ray * 32 + lane] = s;
+    }
 }
 
 // The kernel variants (see Variant): precision, epilogue warps, staggered.
@@ -2113,9 +2159,9 @@ constexpr TcVariant make_variant() {
     return TcVariant{F8 ? MCL_PREC_FP8 : MCL_PREC_BF16, W, S, &k_mlp_tc<F8, W, S>,
                      Variant<F8, W, S>::kThreads, Form<F8>::kSmemBytes, 1};
 }
-template <bool F8, bool S>
+template <bool F8, int W, bool S>
 constexpr TcVariant make_pair_variant() {
-    return TcVariant{F8 ? MCL_PREC_FP8 : MCL_PREC_BF16, 4, S, &k_mlp_tc2<F8, S>, kPairThreads,
+    return TcVariant{F8 ? MCL_PREC_FP8 : MCL_PREC_BF16, W, S, &k_mlp_tc2<F8, W, S>, kPairThreads<W>,
                      PairForm<F8>::kSmemBytes, 2};
 }
 const TcVariant kVariants[] = {
@@ -2124,9 +2170,9 @@ const TcVariant kVariants[] = {
     make_variant<true, 4, true>(),   make_variant<true, 8, true>(),
     TcVariant{MCL_PREC_BF16, 4, true, &k_mlp_tc_split, kSplitThreads, kSplitSmem, 1},
     TcVariant{MCL_PREC_BF16, 4, false, &k_mlp_tc_pipe, kPipeThreads, kPipeSmem, 1},
-    make_pair_variant<false, false>(), make_pair_variant<true, false>(),
-    make_pair_variant<true, true>(),     make_variant<false, 4, true>(),
-    make_variant<false, 8, true>(),      make_pair_variant<false, true>(),
+    make_pair_variant<false, 4, false>(), make_pair_variant<true, 4, false>(),
+    make_pair_variant<true, 8, true>(),  make_variant<false, 4, true>(),
+    make_variant<false, 8, true>(),      make_pair_variant<false, 4, true>(),
 };
 // Fused passes (Params::fuse 1, 2) run on the single-CTA kernel with 4
 // epilogue warps per tile (the fused ray epilogues need one thread per row)
@@ -2136,10 +2182,15 @@ void (*const kFusedKernels[2][2])(Params) = {
     {&k_mlp_tc<true, 4, true, 1>, &k_mlp_tc<true, 4, true, 2>}};
 constexpr int kNumVariants = sizeof(kVariants) / sizeof(kVariants[0]);
 static_assert(kNumVariants == MCL_MLP_VARIANTS, "variant table");
-// untuned choice per precision: 8 epilogue warps per tile, staggered tiles
-// (the autotuner's pick on GB300 at 0.3 M and 2.5 M rows: BF16 about 1.5 %,
-// FP8 about 7 % faster than with 4 warps).
-constexpr int kDefaultVariant[3] = {-1, 12, 5};
+// untuned choice per precision: BF16 the staggered CTA pair, FP8 the
+// staggered single-CTA kernel with 8 epilogue warps per tile (the autotuner's
+// pick on GB300 at 0.3 M and 2.5 M rows; BF16 2.02 against 2.13 ms for the
+// best single-CTA kernel, FP8 1.50 against 1.52 for its pair).
+constexpr int kDefaultVariant[3] = {-1, 13, 5};
+// The failure-injection hook's kernels (it is in the single-CTA kernel).
+constexpr int kHeldVariant[3] = {-1, 12, 5};
+// Point queries (rays of one sample, RayBias interleaved) on the defaults.
+void (*const kPointKernels[2])(Params) = {&k_mlp_tc2<false, 4, true, true>, &k_mlp_tc<true, 8, true, 0, true>};
 // The variant whose launch shape (threads, shared memory) the fused passes'
 // kernels (kFusedKernels: staggered, 4 epilogue warps per tile) share:
 // checked when the map's forms are set up.
@@ -2153,7 +2204,8 @@ struct TcForm {
 struct TcState {
     TcForm bf16, fp8, bf16_split;
     float* aux = nullptr;      // fp32 biases, scales and small heads
-    float* ray_bias = nullptr; // [max_rays][128]
+    float* ray_bias = nullptr; // per ray 128 values (RayBias)
+    int ray_bias_step = 1;
     int* abort_flag = nullptr;
     EpiConsts ec;              // copied into every launch's parameter block
     const float* beta_g = nullptr;
@@ -2412,7 +2464,7 @@ int mlp_tc_prepare(mcl_map* m, const float* blob) {
         (rc = cuda_check(cudaMalloc(&st->aux, aux.size() * 4), "cudaMalloc(tc aux)")) ||
         (rc = cuda_check(cudaMemcpy(st->aux, aux.data(), aux.size() * 4, cudaMemcpyHostToDevice),
                          "upload tc aux")) ||
-        (rc = cuda_check(cudaMalloc(&st->ray_bias, (size_t)m->cfg.max_rays * 128 * 4), "ray bias")) ||
+        (rc = cuda_check(cudaMalloc(&st->ray_bias, ((size_t)m->cfg.max_rays + 31) / 32 * 32 * 128 * 4), "ray bias")) ||
         (rc = cuda_check(cudaMalloc(&st->abort_flag, sizeof(int)), "abort flag")))
         return rc;
     st->beta_g = st->aux + o_beta;
@@ -2431,6 +2483,11 @@ int mlp_tc_prepare(mcl_map* m, const float* blob) {
                                                   (int)v.smem),
                              "smem attribute")))
             return rc;
+    for (int f8 = 0; f8 < 2; ++f8)
+        if ((rc = cuda_check(cudaFuncSetAttribute(kPointKernels[f8], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                  (int)kVariants[kDefaultVariant[f8 + 1]].smem),
+                             "smem attribute (points)")))
+            return rc;
     // the fused kernels launch with their shape variant's threads and smem
     if (kVariants[kFusedVariant[MCL_PREC_BF16]].fn != &k_mlp_tc<false, 4, true> ||
         kVariants[kFusedVariant[MCL_PREC_FP8]].fn != &k_mlp_tc<true, 4, true>)
@@ -2446,9 +2503,9 @@ int mlp_tc_prepare(mcl_map* m, const float* blob) {
         // persistent grid of the pair kernels: every pair resident at once
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)(st->n_sm & ~1));
-        cfg.blockDim = dim3(kPairThreads);
+        cfg.blockDim = dim3(kPairThreads<8>);
         cfg.dynamicSmemBytes = PairForm<false>::kSmemBytes;
-        if ((rc = cuda_check(cudaOccupancyMaxActiveClusters(&st->max_pairs, &k_mlp_tc2<false, false>, &cfg),
+        if ((rc = cuda_check(cudaOccupancyMaxActiveClusters(&st->max_pairs, &k_mlp_tc2<true, 8, true>, &cfg),
                              "pair occupancy")))
             return rc;
         st->max_pairs = std::min(st->max_pairs, st->n_sm / 2);
@@ -2482,16 +2539,24 @@ bool mlp_tc_available(const mcl_map* m, int precision) {
 }
 
 cudaError_t mlp_tc_ray_bias(mcl_map* m, const float* gd, int n_rays, const int* n_rays_dev,
-                            cudaStream_t s) {
+                            cudaStream_t s, bool points, int precision) {
     TcState* st = (TcState*)m->tc_aux;
-    const long n = (long)n_rays * 128;
+    // (the other kernel variants read the rays one after the other)
+    if (precision != MCL_PREC_FP32 && st->variant[precision] != kDefaultVariant[precision]) points = false;
+    st->ray_bias_step = points ? 32 : 1;
     note_launch();
-    k_ray_bias<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(gd, n_rays, n_rays_dev, st->Wd,
-                                                           st->bprime, st->ray_bias);
+    float4* out = reinterpret_cast<float4*>(st->ray_bias);
+    if (points)
+        k_ray_bias<true><<<(unsigned)(((long)n_rays + 31) / 32), 256, 0, s>>>(gd, n_rays, n_rays_dev, st->Wd, st->bprime, out);
+    else
+        k_ray_bias<false><<<(unsigned)(((long)n_rays + 7) / 8), 256, 0, s>>>(gd, n_rays, n_rays_dev, st->Wd, st->bprime, out);
     return cudaGetLastError();
 }
 
-const float* mlp_tc_ray_bias_buffer(const mcl_map* m) { return ((const TcState*)m->tc_aux)->ray_bias; }
+RayBias mlp_tc_ray_bias_result(const mcl_map* m) {
+    const TcState* st = (const TcState*)m->tc_aux;
+    return RayBias{st->ray_bias, st->ray_bias_step};
+}
 
 static cudaError_t mlp_tc_variant(mcl_map* m, int precision, int variant, const Ray* rays,
                                   const float* z, int S, int n_rays, const int* rows_dev,
@@ -2543,7 +2608,7 @@ static cudaError_t mlp_tc_variant(mcl_map* m, int precision, int variant, const 
     p.alpha_sigma = st->alpha_sigma;
     p.s_gx = st->s_gx;
     p.b_sigma = st->b_sigma;
-    p.ray_bias = st->ray_bias;
+    p.ray_bias = mlp_tc_ray_bias_result(m);
     p.b_out0 = st->b_out[0];
     p.b_out1 = st->b_out[1];
     p.b_out2 = st->b_out[2];
@@ -2580,7 +2645,7 @@ static cudaError_t mlp_tc_variant(mcl_map* m, int precision, int variant, const 
         --st->hold_launches;
         p.hold_weights = 1;
         p.wait_ns = st->hold_wait_ns;
-        vsel = fuse ? kFusedVariant[precision] : kDefaultVariant[precision];
+        vsel = fuse ? kFusedVariant[precision] : kHeldVariant[precision];
         p.wblocks = precision == MCL_PREC_FP8 ? st->fp8.wblocks : st->bf16.wblocks;
     }
     cudaError_t e = cudaMemsetAsync(st->abort_flag, 0, sizeof(int), s);
@@ -2588,7 +2653,9 @@ static cudaError_t mlp_tc_variant(mcl_map* m, int precision, int variant, const 
     // persistent grid: one CTA per SM at most, one per work unit (a pair of
     // tiles, a single tile for the pipelined kernel, 512 rows for a CTA pair)
     const TcVariant& v = kVariants[vsel];
-    void (*fn)(Params) = fuse ? kFusedKernels[precision == MCL_PREC_FP8][fuse->mode - 1] : v.fn;
+    void (*fn)(Params) = fuse ? kFusedKernels[precision == MCL_PREC_FP8][fuse->mode - 1]
+                         : st->ray_bias_step == 32 && !p.hold_weights ? kPointKernels[precision == MCL_PREC_FP8]
+                                                   : v.fn;
     long long grid;
     if (v.cluster == 2) {
         const long long units = (p.M + 511) / 512;

@@ -141,8 +141,6 @@ __device__ __forceinline__ uint32_t named_bar_popc(uint32_t id, uint32_t nthread
 }
 
 // ---- CTA pairs (clusters of 2) ----------------------------------------------
-// Waits on barriers that a peer CTA arrives on (release at cluster scope)
-// acquire at cluster scope; otherwise as mbar_wait / mbar_wait_sleep.
 __device__ __forceinline__ uint32_t cluster_ctarank() {
     uint32_t r;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -157,52 +155,13 @@ __device__ __forceinline__ uint32_t mapa_shared(uint32_t addr, uint32_t rank) {
     return r;
 }
 
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr)
-                 : "memory");
-}
-
-// As mbar_arrive_cluster with the default release at CTA scope: for arrivals
-// that only tell the peer's tensor core of shared-memory writes already made
-// visible by fence.proxy.async, or of TMEM reads that have completed.  (The
-// cluster-scope release waits for every earlier global and local store.)
+// Arrive on a barrier of a CTA of the cluster (shared::cluster address),
+// release at CTA scope: the arrivals only tell the even CTA's tensor core of
+// shared-memory writes already made visible by fence.proxy.async, or of TMEM
+// reads that have completed.  (A cluster-scope release waits for every
+// earlier global and local store.)
 __device__ __forceinline__ void mbar_arrive_peer(uint32_t cluster_addr) {
     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n"
-        ".reg .pred p;\n"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
-        "selp.u32 %0, 1, 0, p;\n"
-        "}\n"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
-template <bool kSleep>
-__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, volatile int* err,
-                                                  unsigned long long limit_ns = kWaitNs) {
-#pragma unroll 1
-    for (int i = 0; i < (kSleep ? 8 : 32); ++i)
-        if (mbar_try_wait_cluster(bar, parity)) return true;
-    const unsigned long long t0 = globaltimer();
-#pragma unroll 1
-    for (uint32_t it = 1;; ++it) {
-        if (kSleep) __nanosleep(128);
-        if (mbar_try_wait_cluster(bar, parity)) return true;
-        if ((it & (kSleep ? 15u : 63u)) == 0u) {
-            if (err && *err != 0) return false;
-            if (globaltimer() - t0 > limit_ns) {
-                if (err) atomicCAS((int*)err, 0, -4 /* MCL_ERR_TIMEOUT */);
-                return false;
-            }
-        }
-    }
 }
 
 // Every thread of both CTAs of the cluster.
@@ -237,17 +196,6 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
         "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
             dst),
         "l"(reinterpret_cast<uint64_t>(src)), "r"(bytes), "r"(bar)
-        : "memory");
-}
-
-// As bulk_load, into the same shared-memory offset of every CTA of cta_mask
-// in the cluster, completing on the barrier at `bar`'s offset in each.
-__device__ __forceinline__ void bulk_load_mc(uint32_t dst, const void* src, uint32_t bytes,
-                                             uint32_t bar, uint16_t cta_mask) {
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster"
-        " [%0], [%1], %2, [%3], %4;" ::"r"(dst),
-        "l"(reinterpret_cast<uint64_t>(src)), "r"(bytes), "r"(bar), "h"(cta_mask)
         : "memory");
 }
 
@@ -418,28 +366,6 @@ __device__ __forceinline__ void mma_commit2_mc(uint32_t bar, uint16_t cta_mask) 
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
     asm volatile(
         "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-        : "memory");
-}
-
-// Single-CTA MMAs: arrive once on the barrier at shared::cta offset `bar` in
-// each CTA of `cta_mask` when this thread's MMAs issued so far complete.
-__device__ __forceinline__ void mma_commit_mc(uint32_t bar, uint16_t cta_mask) {
-    asm volatile(
-        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64"
-        " [%0], %1;" ::"r"(bar),
-        "h"(cta_mask)
-        : "memory");
-}
-
-// 32 lanes x 16 consecutive 32-bit columns (as tmem_ld32).
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
-          "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]),
-          "=r"(v[14]), "=r"(v[15])
-        : "r"(taddr)
         : "memory");
 }
 
