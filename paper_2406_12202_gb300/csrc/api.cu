@@ -35,6 +35,37 @@ static std::atomic<long long> g_launches{0};
 
 void note_launch(int n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 
+int Scratch::take(mcl_map* m) {
+    size_t total = 0;
+    for (const Piece& q : pieces_) total += (q.bytes + 255) & ~(size_t)255;
+    m_ = m;
+    char* base;
+    if (total <= kScratchKeep) {
+        if (m->scratch_bytes < total) {
+            if (m->scratch) cudaFree(m->scratch);
+            m->scratch = nullptr;
+            m->scratch_bytes = 0;
+            const int rc = cuda_check(cudaMalloc(&m->scratch, total), "scratch");
+            if (rc) return rc;
+            m->scratch_bytes = total;
+        }
+        base = (char*)m->scratch;
+    } else {
+        const int rc = cuda_check(cudaMalloc(&own_, total), "scratch");
+        if (rc) return rc;
+        base = (char*)own_;
+    }
+    for (const Piece& q : pieces_) {
+        *q.p = base;
+        base += (q.bytes + 255) & ~(size_t)255;
+    }
+    return MCL_OK;
+}
+
+Scratch::~Scratch() {
+    if (own_) cudaFree(own_);
+}
+
 // Per-phase timing: an event pair recorded on the call's stream around a
 // phase when the map's profiling flag is set.
 static cudaEvent_t ev_get(mcl_map* m) {
@@ -106,7 +137,7 @@ static void free_map(mcl_map* m) {
                     m->logw64, m->cdf, m->status, m->act0, m->act1, m->gxbuf,
                     m->loop.plan, m->loop.qs, m->loop.n0, (void*)m->loop.imgs, m->loop.pix,
                     m->loop.P_next, m->loop.w, m->loop.mask, m->loop.idx, m->prop_w,
-                    m->prop_packed, m->prop_abort};
+                    m->prop_packed, m->prop_abort, m->scratch};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     delete m;

@@ -1,10 +1,9 @@
 // fit.cu -- fitting the NeRF map's FP32 weights to samples of a field: points
 // x with view directions and targets (density, r, g, b), loss
 //   L = mean over points of  w_sigma (sigma_raw(x) - sigma_t)^2 + |rgb(x, d) - rgb_t|^2,
-// minimised by Adam with the library's own kernels: the plain FP32 form's
-// forward (gamma(x), SGEMM layers, heads) with every layer's output kept, a
-// backward pass of SGEMMs on transposed weights with ReLU masks, and weight
-// gradients summed over the batch in a fixed order (the same inputs give the
+// minimised by Adam with the library's own kernels: the SIMT FP32 forward
+// (gamma(x), SGEMM layers, heads) with every layer's output kept, a backward
+// pass of SGEMMs with the ReLU masks in their epilogue, and weight gradients summed over the batch in a fixed order (the same inputs give the
 // same weights).  The map's tensor-core forms are rebuilt from the fitted
 // weights.  This stands in for training a map on images (Eq. 2, out of
 // scope): it gives maps of analytic scenes whose weights the library itself
@@ -37,55 +36,46 @@ struct FitBuf {
     float* dlog = nullptr;      // [B][4]: d rgb logits, d sigma
     float* part = nullptr;      // partial weight gradients
     float* partb = nullptr;     // partial bias gradients
-    float* wt = nullptr;        // transposed weights [256][256]
-    float* zeros = nullptr;     // [256]
     double* lpart = nullptr;    // per-block loss partials
     double* loss = nullptr;
     float* grad = nullptr;      // [w32_n] gradient in the padded layout
     float *m1 = nullptr, *m2 = nullptr;   // Adam moments
 };
 
-void free_buf(FitBuf& b) {
-    void* ptrs[] = {b.x, b.dir, b.tgt, b.rays, b.gd, b.z, b.gx, b.h, b.feat, b.hid, b.out, b.dA,
-                    b.dB, b.dhid, b.dlog, b.part, b.partb, b.wt, b.zeros, b.lpart, b.loss, b.grad,
-                    b.m1, b.m2};
-    for (void* p : ptrs)
-        if (p) cudaFree(p);
-    b = FitBuf{};
-}
-
-int alloc_buf(mcl_map* m, FitBuf& b, long B, bool adam) {
+int alloc_buf(mcl_map* m, Scratch& sc, FitBuf& b, long B, bool adam) {
     b.B = B;
     const long nchunk = (B + kWgRows - 1) / kWgRows;
-    struct {
-        void** p;
-        size_t bytes;
-    } a[] = {
-        {(void**)&b.x, sizeof(float) * 3 * B},        {(void**)&b.dir, sizeof(float) * 3 * B},
-        {(void**)&b.tgt, sizeof(float) * 4 * B},      {(void**)&b.rays, sizeof(Ray) * B},
-        {(void**)&b.gd, sizeof(float) * kGdPad * B},  {(void**)&b.z, sizeof(float) * B},
-        {(void**)&b.gx, sizeof(float) * kGxPad * B},  {(void**)&b.h, sizeof(float) * 8 * kWidth * B},
-        {(void**)&b.feat, sizeof(float) * kWidth * B}, {(void**)&b.hid, sizeof(float) * kWidth * B},
-        {(void**)&b.out, sizeof(float4) * B},          {(void**)&b.dA, sizeof(float) * kWidth * B},
-        {(void**)&b.dB, sizeof(float) * kWidth * B},   {(void**)&b.dhid, sizeof(float) * kWidth * B},
-        {(void**)&b.dlog, sizeof(float) * 4 * B},
-        {(void**)&b.part, sizeof(float) * nchunk * kWidth * (kWidth + kGxPad)},
-        {(void**)&b.partb, sizeof(float) * nchunk * kWidth},
-        {(void**)&b.wt, sizeof(float) * kWidth * kWidth}, {(void**)&b.zeros, sizeof(float) * kWidth},
-        {(void**)&b.lpart, sizeof(double) * ((B + 255) / 256)}, {(void**)&b.loss, sizeof(double)},
-        {(void**)&b.grad, sizeof(float) * m->w32_n},
-    };
-    int rc;
-    for (auto& e : a)
-        if ((rc = cuda_check(cudaMalloc(e.p, e.bytes), "fit buffers"))) return rc;
+    sc.add(&b.x, sizeof(float) * 3 * B);
+    sc.add(&b.dir, sizeof(float) * 3 * B);
+    sc.add(&b.tgt, sizeof(float) * 4 * B);
+    sc.add(&b.rays, sizeof(Ray) * B);
+    sc.add(&b.gd, sizeof(float) * kGdPad * B);
+    sc.add(&b.z, sizeof(float) * B);
+    sc.add(&b.gx, sizeof(float) * kGxPad * B);
+    sc.add(&b.h, sizeof(float) * 8 * kWidth * B);
+    sc.add(&b.feat, sizeof(float) * kWidth * B);
+    sc.add(&b.hid, sizeof(float) * kWidth * B);
+    sc.add(&b.out, sizeof(float4) * B);
+    sc.add(&b.dA, sizeof(float) * kWidth * B);
+    sc.add(&b.dB, sizeof(float) * kWidth * B);
+    sc.add(&b.dhid, sizeof(float) * kWidth * B);
+    sc.add(&b.dlog, sizeof(float) * 4 * B);
+    sc.add(&b.part, sizeof(float) * nchunk * kWidth * (kWidth + kGxPad));
+    sc.add(&b.partb, sizeof(float) * nchunk * kWidth);
+    sc.add(&b.lpart, sizeof(double) * ((B + 255) / 256));
+    sc.add(&b.loss, sizeof(double));
+    sc.add(&b.grad, sizeof(float) * m->w32_n);
     if (adam) {
-        if ((rc = cuda_check(cudaMalloc(&b.m1, sizeof(float) * m->w32_n), "fit moments")) ||
-            (rc = cuda_check(cudaMalloc(&b.m2, sizeof(float) * m->w32_n), "fit moments")))
-            return rc;
-        cudaMemset(b.m1, 0, sizeof(float) * m->w32_n);
-        cudaMemset(b.m2, 0, sizeof(float) * m->w32_n);
+        sc.add(&b.m1, sizeof(float) * m->w32_n);
+        sc.add(&b.m2, sizeof(float) * m->w32_n);
     }
-    cudaMemset(b.zeros, 0, sizeof(float) * kWidth);
+    int rc;
+    if ((rc = sc.take(m))) return rc;
+    if (adam) {
+        if ((rc = cuda_check(cudaMemset(b.m1, 0, sizeof(float) * m->w32_n), "clear moments")) ||
+            (rc = cuda_check(cudaMemset(b.m2, 0, sizeof(float) * m->w32_n), "clear moments")))
+            return rc;
+    }
     return MCL_OK;
 }
 
@@ -167,82 +157,150 @@ __global__ void k_fit_dtop(float* __restrict__ d, const float* __restrict__ dlog
     d[t] = h8[t] > 0.f ? v : 0.f;
 }
 
-__global__ void k_fit_mask(float* __restrict__ d, const float* __restrict__ h, long n) {
-    const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < n && !(h[t] > 0.f)) d[t] = 0.f;
-}
-
-// Wt[k][o] = W[o][k] for o < n_out, k < n_in (W row stride ldw).
-__global__ void k_fit_transpose(const float* __restrict__ W, int ldw, int n_out, int n_in,
-                                float* __restrict__ Wt) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n_out * n_in) return;
-    const int k = t / n_out, o = t - k * n_out;
-    Wt[t] = W[o * ldw + k];
-}
-
 // Partial weight gradients of one row chunk:
 //   part[c][o][k] = sum_{rows p of chunk c} dY[p][o] X[p][k],  X = [X1 | X2],
 //   partb[c][o] = sum_p dY[p][o].
-// 64 x 64 outputs per block (256 threads, 4 x 4 each), rows staged 16 at a
-// time in shared memory; every sum runs over the chunk's rows in order.
-__global__ __launch_bounds__(256) void k_wgrad(const float* __restrict__ dY, int ldy, int N,
+// 64 x 64 outputs per block, 8 x 4 per thread (three 16-byte loads for 16
+// packed FMAs on pairs of outputs); the rows pass through shared memory 16 at
+// a time, the next 32 on their way (cp.async).  Every sum is one chain of
+// FMAs over the chunk's rows in order.  N and K1 are multiples of 64, K2 of
+// 32, rows 16-byte aligned.  Bound by the FMA lanes; with 16 chunks (16,384
+// rows) there are 256 blocks of 4 warps for 152 SMs.
+constexpr int kWgStage = 16, kWgBufs = 4;
+
+__device__ __forceinline__ void cp_async16(float* dst, const float* src, bool in) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
+                 "l"(src), "r"(in ? 16 : 0)
+                 : "memory");
+}
+
+__global__ __launch_bounds__(128) void k_wgrad(const float* __restrict__ dY, int ldy, int N,
                                                const float* __restrict__ X1, int ld1, int K1,
                                                const float* __restrict__ X2, int ld2, int K2,
                                                long rows, float* __restrict__ part,
                                                float* __restrict__ partb) {
-    __shared__ float As[16][kWgTile + 4];
-    __shared__ float Bs[16][kWgTile + 4];
+    __shared__ __align__(16) float As[kWgBufs][kWgStage][kWgTile];
+    __shared__ __align__(16) float Bs[kWgBufs][kWgStage][kWgTile];
     const int K = K1 + K2;
     const int o0 = blockIdx.x * kWgTile, k0 = blockIdx.y * kWgTile, c = blockIdx.z;
     const long p0 = (long)c * kWgRows, p1 = min(rows, p0 + kWgRows);
-    const int t = threadIdx.x, ty = t >> 4, tx = t & 15;
-    float acc[4][4] = {};
-    float accb[4] = {0.f, 0.f, 0.f, 0.f};
-    for (long pb = p0; pb < p1; pb += 16) {
-        // stage 16 rows: thread t loads element (row t / 16, 4 columns (t % 16) * 4)
-        {
-            const int r = t >> 4, cc = (t & 15) * 4;
-            const long p = pb + r;
+    const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
+    // the block's columns lie in one of X1, X2 (K1 is a multiple of the tile)
+    const float* X = k0 < K1 ? X1 + k0 : X2 + (k0 - K1);
+    const int ldx = k0 < K1 ? ld1 : ld2;
+    auto load = [&](int st) {   // stage st (a group is committed past the end, too)
+        const long pb = p0 + (long)st * kWgStage;
+        const int buf = st % kWgBufs;
+        if (pb < p1) {
+#pragma unroll
+            for (int q = 0; q < kWgStage * kWgTile / 4 / 128; ++q) {
+                const int r = (t >> 4) + 8 * q, cc = (t & 15) * 4;
+                const bool in = pb + r < p1;
+                const long p = in ? pb + r : p0;
+                cp_async16(&As[buf][r][cc], dY + p * ldy + o0 + cc, in);
+                const bool ink = in && k0 + cc < K;
+                cp_async16(&Bs[buf][r][cc], ink ? X + p * ldx + cc : X, ink);
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    float2 acc[4][4], accb[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        accb[i] = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
+    }
+    load(0);
+    load(1);
+    load(2);
+    int st = 0;
+    for (long pb = p0; pb < p1; pb += kWgStage, ++st) {
+        asm volatile("cp.async.wait_group 2;" ::: "memory");
+        __syncthreads();     // stage st has landed; stage st - 1 has been read
+        load(st + 3);
+        const int cur = st % kWgBufs, n = (int)min((long)kWgStage, p1 - pb);
+        auto row = [&](int r) {
+            const float4 a0 = *reinterpret_cast<const float4*>(&As[cur][r][ty * 8]);
+            const float4 a1 = *reinterpret_cast<const float4*>(&As[cur][r][ty * 8 + 4]);
+            const float4 x = *reinterpret_cast<const float4*>(&Bs[cur][r][tx * 4]);
+            const float2 a[4] = {make_float2(a0.x, a0.y), make_float2(a0.z, a0.w),
+                                 make_float2(a1.x, a1.y), make_float2(a1.z, a1.w)};
+            const float xv[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                const int o = o0 + cc + j, k = k0 + cc + j;
-                As[r][cc + j] = (p < p1 && o < N) ? dY[p * ldy + o] : 0.f;
-                float xv = 0.f;
-                if (p < p1 && k < K) xv = k < K1 ? X1[p * ld1 + k] : X2[p * ld2 + (k - K1)];
-                Bs[r][cc + j] = xv;
+                const float2 xj = make_float2(xv[j], xv[j]);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) acc[i][j] = __ffma2_rn(a[i], xj, acc[i][j]);
             }
+            if (blockIdx.y == 0)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) accb[i] = __fadd2_rn(accb[i], a[i]);
+        };
+        if (n == kWgStage) {
+#pragma unroll
+            for (int r = 0; r < kWgStage; ++r) row(r);
+        } else {
+            for (int r = 0; r < n; ++r) row(r);
         }
-        __syncthreads();
-#pragma unroll
-        for (int r = 0; r < 16; ++r) {
-            float a[4], b[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                a[i] = As[r][ty * 4 + i];
-                b[i] = Bs[r][tx * 4 + i];
-            }
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-                accb[i] += a[i];
-            }
-        }
-        __syncthreads();
     }
     float* pc = part + (size_t)c * N * K;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int o = o0 + ty * 4 + i;
-        if (o >= N) continue;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int k = k0 + tx * 4 + j;
-            if (k < K) pc[(size_t)o * K + k] = acc[i][j];
-        }
-        if (blockIdx.y == 0 && tx == 0) partb[(size_t)c * N + o] = accb[i];
+    for (int i = 0; i < 8; ++i) {
+        const int o = o0 + ty * 8 + i;
+        const float2* ar = acc[i >> 1];
+        const float4 v = (i & 1) ? make_float4(ar[0].y, ar[1].y, ar[2].y, ar[3].y)
+                                 : make_float4(ar[0].x, ar[1].x, ar[2].x, ar[3].x);
+        if (k0 + tx * 4 < K) *reinterpret_cast<float4*>(pc + (size_t)o * K + k0 + tx * 4) = v;
+        if (blockIdx.y == 0 && tx == 0) partb[(size_t)c * N + o] = (i & 1) ? accb[i >> 1].y : accb[i >> 1].x;
     }
+}
+
+// The same for the heads (N <= 4 outputs): 64 input columns per block, a
+// thread per output and column, the rows staged in shared memory 64 at a time.
+__global__ __launch_bounds__(256) void k_wgrad_head(const float* __restrict__ dY, int ldy, int N,
+                                                    const float* __restrict__ X, int ldx, int K,
+                                                    long rows, float* __restrict__ part,
+                                                    float* __restrict__ partb) {
+    __shared__ __align__(16) float xs[2][64][64];
+    __shared__ float ds[2][64][4];
+    const int k0 = blockIdx.x * 64, c = blockIdx.y, t = threadIdx.x, o = t >> 6, kk = t & 63;
+    const long p0 = (long)c * kWgRows, p1 = min(rows, p0 + kWgRows);
+    auto load = [&](long pb, int buf) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int r = (t >> 4) + 16 * q, cc = (t & 15) * 4;
+            const bool in = pb + r < p1 && k0 + cc < K;
+            cp_async16(&xs[buf][r][cc], in ? X + (pb + r) * ldx + k0 + cc : X, in);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        const int r = t & 63, oo = t >> 6;
+        ds[buf][r][oo] = (pb + r < p1 && oo < N) ? dY[(pb + r) * ldy + oo] : 0.f;
+    };
+    float acc = 0.f, accb = 0.f;
+    load(p0, 0);
+    int cur = 0;
+    for (long pb = p0; pb < p1; pb += 64, cur ^= 1) {
+        if (pb + 64 < p1) {
+            load(pb + 64, cur ^ 1);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+        __syncthreads();
+        const int n = (int)min(64l, p1 - pb);
+        if (o < N) {
+#pragma unroll 8
+            for (int r = 0; r < n; ++r) {
+                const float a = ds[cur][r][o];
+                acc = fmaf(a, xs[cur][r][kk], acc);
+                accb += a;
+            }
+        }
+        __syncthreads();
+    }
+    if (o < N && k0 + kk < K) part[((size_t)c * N + o) * K + k0 + kk] = acc;
+    if (o < N && k0 + kk == 0) partb[(size_t)c * N + o] = accb;
 }
 
 // gW[o][k] (row stride ldg) = sum over chunks in order of part[c][o][k];
@@ -269,9 +327,12 @@ cudaError_t wgrad(const FitBuf& b, long n, const float* dY, int ldy, int N, cons
                   float* gb, cudaStream_t s) {
     const int K = K1 + K2;
     const int nchunk = (int)((n + kWgRows - 1) / kWgRows);
-    dim3 grid((N + kWgTile - 1) / kWgTile, (K + kWgTile - 1) / kWgTile, nchunk);
     note_launch(2);
-    k_wgrad<<<grid, 256, 0, s>>>(dY, ldy, N, X1, ld1, K1, X2, ld2, K2, n, b.part, b.partb);
+    if (N <= 4)
+        k_wgrad_head<<<dim3((K + 63) / 64, nchunk), 256, 0, s>>>(dY, ldy, N, X1, ld1, K, n, b.part, b.partb);
+    else
+        k_wgrad<<<dim3(N / kWgTile, (K + kWgTile - 1) / kWgTile, nchunk), 128, 0, s>>>(
+            dY, ldy, N, X1, ld1, K1, X2, ld2, K2, n, b.part, b.partb);
     k_wgrad_reduce<<<(N * K + 255) / 256, 256, 0, s>>>(b.part, b.partb, nchunk, N, K, gW, ldg, gb);
     return cudaGetLastError();
 }
@@ -322,20 +383,12 @@ cudaError_t loss_and_grad(mcl_map* m, const FitBuf& b, long n, float wsig, float
     if ((e = wgrad(b, n, b.dhid, kWidth, kRgbW, b.feat, kWidth, kWidth, b.gd, kGdPad, kGdPad,
                    off(L[10].W), L[10].k_pad, off(L[10].b), s)))
         return e;
-    note_launch();
-    k_fit_transpose<<<(kRgbW * kWidth + 255) / 256, 256, 0, s>>>(L[10].W, L[10].k_pad, kRgbW, kWidth, b.wt);
-    if ((e = fp32_gemm(b.dhid, kWidth, kRgbW, nullptr, 0, 0, 0, 1, b.wt, b.zeros, kWidth, b.dA, kWidth,
-                       (int)n, false, s)))
-        return e;
+    if ((e = fp32_gemm_back(b.dhid, kRgbW, L[10].W, L[10].k_pad, nullptr, b.dA, (int)n, s))) return e;
     // feature layer (linear 256 x 256), then d h8 through it
     if ((e = wgrad(b, n, b.dA, kWidth, kWidth, H(7), kWidth, kWidth, nullptr, 0, 0, off(L[9].W),
                    L[9].k_pad, off(L[9].b), s)))
         return e;
-    note_launch();
-    k_fit_transpose<<<(kWidth * kWidth + 255) / 256, 256, 0, s>>>(L[9].W, L[9].k_pad, kWidth, kWidth, b.wt);
-    if ((e = fp32_gemm(b.dA, kWidth, kWidth, nullptr, 0, 0, 0, 1, b.wt, b.zeros, kWidth, b.dB, kWidth,
-                       (int)n, false, s)))
-        return e;
+    if ((e = fp32_gemm_back(b.dA, kWidth, L[9].W, L[9].k_pad, nullptr, b.dB, (int)n, s))) return e;
     // density head (1 x 256) gradient from d sigma (column 3 of dlog)
     if ((e = wgrad(b, n, b.dlog + 3, 4, 1, H(7), kWidth, kWidth, nullptr, 0, 0, off(L[8].W),
                    L[8].k_pad, off(L[8].b), s)))
@@ -357,13 +410,7 @@ cudaError_t loss_and_grad(mcl_map* m, const FitBuf& b, long n, float wsig, float
                       L[l].k_pad, off(L[l].b), s);
         if (e) return e;
         if (l == 0) break;
-        note_launch(2);
-        k_fit_transpose<<<(kWidth * kWidth + 255) / 256, 256, 0, s>>>(L[l].W, L[l].k_pad, kWidth, kWidth,
-                                                                     b.wt);
-        if ((e = fp32_gemm(cur, kWidth, kWidth, nullptr, 0, 0, 0, 1, b.wt, b.zeros, kWidth, nxt, kWidth,
-                           (int)n, false, s)))
-            return e;
-        k_fit_mask<<<(unsigned)((n * kWidth + 255) / 256), 256, 0, s>>>(nxt, H(l - 1), n * kWidth);
+        if ((e = fp32_gemm_back(cur, kWidth, L[l].W, L[l].k_pad, H(l - 1), nxt, (int)n, s))) return e;
         std::swap(cur, nxt);
     }
     return cudaGetLastError();
@@ -390,38 +437,49 @@ int map_download(mcl_map* m, float* host_blob) {
     return MCL_OK;
 }
 
+// Gradient in the padded layer layout -> blob layout (one layer per grid row).
+struct Unpad {
+    int src_w[12], src_b[12], dst[12], fin[12], fout[12], ld[12];
+};
+__global__ void k_unpad(const float* __restrict__ g, Unpad u, float* __restrict__ out) {
+    const int l = blockIdx.y, nw = u.fin[l] * u.fout[l];
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < nw) out[u.dst[l] + t] = g[u.src_w[l] + (t / u.fin[l]) * u.ld[l] + t % u.fin[l]];
+    else if (t < nw + u.fout[l]) out[u.dst[l] + t] = g[u.src_b[l] + t - nw];
+}
+
 int map_loss_grad(mcl_map* m, const float* d_x, const float* d_dir, const float* d_target, int n,
                   float sigma_weight, double* d_loss, float* d_grad, cudaStream_t s) {
     FitBuf b;
-    int rc = alloc_buf(m, b, n, false);
-    if (!rc) {
-        note_launch();
-        k_fit_gather<<<(n + 255) / 256, 256, 0, s>>>(d_x, d_dir, d_target, nullptr, 0, n, b.x, b.dir, b.tgt);
-        rc = cuda_check(cudaMemsetAsync(b.grad, 0, sizeof(float) * m->w32_n, s), "clear grad");
-    }
+    Scratch sc;
+    int rc = alloc_buf(m, sc, b, n, false);
+    if (rc) return rc;
+    note_launch();
+    k_fit_gather<<<(n + 255) / 256, 256, 0, s>>>(d_x, d_dir, d_target, nullptr, 0, n, b.x, b.dir, b.tgt);
+    rc = cuda_check(cudaMemsetAsync(b.grad, 0, sizeof(float) * m->w32_n, s), "clear grad");
     if (!rc) rc = cuda_check(loss_and_grad(m, b, n, sigma_weight, nullptr, s), "loss and gradient");
+    if (!rc) {
+        Unpad u;
+        blob_layer_shapes(u.fin, u.fout);
+        int dst = 0, most = 0;
+        for (int l = 0; l < 12; ++l) {
+            u.src_w[l] = (int)(m->L[l].W - m->w32);
+            u.src_b[l] = (int)(m->L[l].b - m->w32);
+            u.ld[l] = m->L[l].k_pad;
+            u.dst[l] = dst;
+            const int size = u.fin[l] * u.fout[l] + u.fout[l];
+            dst += size;
+            most = std::max(most, size);
+        }
+        note_launch();
+        k_unpad<<<dim3((most + 255) / 256, 12), 256, 0, s>>>(b.grad, u, d_grad);
+        rc = cuda_check(cudaGetLastError(), "gradient layout");
+    }
     if (!rc) rc = cuda_check(cudaMemcpyAsync(d_loss, b.loss, sizeof(double), cudaMemcpyDeviceToDevice, s),
                              "copy loss");
-    if (!rc) rc = cuda_check(cudaStreamSynchronize(s), "loss sync");
-    if (!rc) {
-        // gradient in the blob layout: the same unpadding as the weights
-        int fin[12], fout[12];
-        blob_layer_shapes(fin, fout);
-        std::vector<float> g(m->w32_n), out;
-        rc = cuda_check(cudaMemcpy(g.data(), b.grad, sizeof(float) * m->w32_n, cudaMemcpyDeviceToHost),
-                        "download grad");
-        for (int l = 0; l < 12 && !rc; ++l) {
-            const size_t oW = m->L[l].W - m->w32, ob = m->L[l].b - m->w32;
-            for (int o = 0; o < fout[l]; ++o)
-                for (int i = 0; i < fin[l]; ++i) out.push_back(g[oW + (size_t)o * m->L[l].k_pad + i]);
-            for (int o = 0; o < fout[l]; ++o) out.push_back(g[ob + o]);
-        }
-        if (!rc)
-            rc = cuda_check(cudaMemcpy(d_grad, out.data(), sizeof(float) * out.size(), cudaMemcpyHostToDevice),
-                            "upload grad");
-    }
-    free_buf(b);
-    return rc;
+    // (also after an error: the scratch may be freed or used again)
+    const int rs = cuda_check(cudaStreamSynchronize(s), "loss sync");
+    return rc ? rc : rs;
 }
 
 int fit_map(mcl_map* m, const float* d_x, const float* d_dir, const float* d_target, int n,
@@ -429,8 +487,9 @@ int fit_map(mcl_map* m, const float* d_x, const float* d_dir, const float* d_tar
     const long B = std::min(n, cfg.batch);
     FitBuf b;
     int* perm_d = nullptr;
-    int rc = alloc_buf(m, b, B, true);
-    if (!rc) rc = cuda_check(cudaMalloc(&perm_d, sizeof(int) * n), "fit permutation");
+    Scratch sc;
+    sc.add(&perm_d, sizeof(int) * n);
+    int rc = alloc_buf(m, sc, b, B, true);
     std::mt19937_64 rng(cfg.seed);
     std::vector<int> perm(n);
     for (int i = 0; i < n; ++i) perm[i] = i;
@@ -466,10 +525,8 @@ int fit_map(mcl_map* m, const float* d_x, const float* d_dir, const float* d_tar
                                         (float)(1.0 - c1), (float)(1.0 - c2), s),
                             "fit adam");
     }
-    if (!rc) rc = cuda_check(cudaStreamSynchronize(s), "fit sync");
-    if (perm_d) cudaFree(perm_d);
-    free_buf(b);
-    return rc;
+    const int rs = cuda_check(cudaStreamSynchronize(s), "fit sync");
+    return rc ? rc : rs;
 }
 
 }  // namespace mcl

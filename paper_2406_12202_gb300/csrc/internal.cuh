@@ -111,6 +111,9 @@ struct mcl_map {
     float* act1 = nullptr;
     float* gxbuf = nullptr;
     int chunk_rows = 0;
+    // scratch of the gradient entry points (Scratch below): kept between calls
+    void* scratch = nullptr;
+    size_t scratch_bytes = 0;
     // per-phase timing (host side)
     struct Mark {
         int phase;
@@ -140,6 +143,30 @@ namespace mcl {
 int fail(int code, const char* fmt, ...);
 void clear_error();
 int cuda_check(cudaError_t e, const char* what);
+// Scratch of one synchronous training or gradient call: one block of device
+// memory cut into pieces.  Up to kScratchKeep bytes stay with the map for its
+// next call (a map is used by one stream at a time); a larger block is freed
+// when the call returns.
+constexpr size_t kScratchKeep = (size_t)1 << 30;
+class Scratch {
+public:
+    // registers *p for n bytes (before take)
+    template <class T>
+    void add(T** p, size_t bytes) {
+        pieces_.push_back({(void**)p, bytes});
+    }
+    int take(mcl_map* m);     // allocates or reuses the block and sets the pieces
+    ~Scratch();
+
+private:
+    struct Piece {
+        void** p;
+        size_t bytes;
+    };
+    std::vector<Piece> pieces_;
+    mcl_map* m_ = nullptr;
+    void* own_ = nullptr;     // a block that is not the map's
+};
 // Count of kernels launched by the library (api.cu).
 void note_launch(int n = 1);
 
@@ -188,6 +215,10 @@ cudaError_t mlp_fp32_simt(mcl_map* m, const Ray* rays, const float* z, int S, in
 cudaError_t fp32_gemm(const float* A1, int lda1, int K1, const float* A2, int lda2, int K2,
                       long a2_off, int a2_div, const float* W, const float* bias, int n_out,
                       float* C, int ldc, int M, bool relu, cudaStream_t s);
+// dX [M, 256] = dY [M, n_out] (row stride 256) W, W [n_out][ldw] (the first 256
+// columns); zero where mask [M, 256] (optional) is not positive.
+cudaError_t fp32_gemm_back(const float* dY, int n_out, const float* W, int ldw, const float* mask,
+                           float* dX, int M, cudaStream_t s);
 cudaError_t fp32_pe(const Ray* rays, const float* z, int n, float* gx, cudaStream_t s);
 cudaError_t fp32_heads(const float* h, const LayerF32& sigma, const float* hid, const LayerF32& rgb,
                        int n, float4* out, cudaStream_t s);

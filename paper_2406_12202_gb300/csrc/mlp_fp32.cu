@@ -65,13 +65,16 @@ __global__ void k_pe_xyz(const Ray* __restrict__ rays, const float* __restrict__
 // 16: while the threads multiply one, the next is loaded from global memory
 // into registers and stored into the other buffer, so each k-tile costs one
 // barrier.  Every output accumulates its products in ascending k with one
-// FMA each.
-template <bool RELU>
+// FMA each.  WT (the backward pass): W is stored the other way round ([K1 +
+// K2][N], row stride ldw), there is no bias, and outputs become zero where
+// mask (optional, [M, N], row stride ldc) is not positive.
+template <bool RELU, bool WT>
 __global__ __launch_bounds__(256, 2) void k_sgemm(const float* __restrict__ A1, int lda1, int K1,
                                                const float* __restrict__ A2, int lda2, int K2,
                                                long a2_off, int a2_div,
-                                               const float* __restrict__ W,
+                                               const float* __restrict__ W, int ldw,
                                                const float* __restrict__ bias,
+                                               const float* __restrict__ mask,
                                                float* __restrict__ C, int ldc, int M,
                                                const int* __restrict__ rows_dev, long r0) {
     constexpr int BM = 128, BN = 128, BK = 16, PAD = 4;
@@ -94,13 +97,13 @@ __global__ __launch_bounds__(256, 2) void k_sgemm(const float* __restrict__ A1, 
 #pragma unroll
         for (int j = 0; j < 8; ++j) acc[i][j] = make_float2(0.f, 0.f);
     float4 ra[2], rb[2];
-    auto load = [&](int k0) {
+    auto load = [&](int k0, int buf) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int row = m0 + lr + h * 64;
             float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
             if (row < M) {
-                if (k0 < K1) {
+                if (WT || k0 < K1) {
                     v = *reinterpret_cast<const float4*>(A1 + (size_t)row * lda1 + k0 + lk);
                 } else {
                     const long r2 = ((long)row + a2_off) / a2_div;
@@ -108,8 +111,18 @@ __global__ __launch_bounds__(256, 2) void k_sgemm(const float* __restrict__ A1, 
                 }
             }
             ra[h] = v;
-            const int nr = n0 + lr + h * 64;
-            rb[h] = *reinterpret_cast<const float4*>(W + (size_t)nr * K + k0 + lk);
+            if constexpr (WT) {
+                // row k0 + (tid / 32) + 8 h of W, four columns, straight to
+                // the other buffer (it was last read before the barrier)
+                const int r = (tid >> 5) + 8 * h, cc = 4 * (tid & 31);
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                                 (uint32_t)__cvta_generic_to_shared(&Bs[buf][r][cc])),
+                             "l"(W + (size_t)(k0 + r) * ldw + n0 + cc)
+                             : "memory");
+            } else {
+                const int nr = n0 + lr + h * 64;
+                rb[h] = *reinterpret_cast<const float4*>(W + (size_t)nr * K + k0 + lk);
+            }
         }
     };
     auto store = [&](int buf) {
@@ -118,17 +131,20 @@ __global__ __launch_bounds__(256, 2) void k_sgemm(const float* __restrict__ A1, 
             const int c = lr + h * 64;
             As[buf][lk + 0][c] = ra[h].x; As[buf][lk + 1][c] = ra[h].y;
             As[buf][lk + 2][c] = ra[h].z; As[buf][lk + 3][c] = ra[h].w;
-            Bs[buf][lk + 0][c] = rb[h].x; Bs[buf][lk + 1][c] = rb[h].y;
-            Bs[buf][lk + 2][c] = rb[h].z; Bs[buf][lk + 3][c] = rb[h].w;
+            if constexpr (!WT) {
+                Bs[buf][lk + 0][c] = rb[h].x; Bs[buf][lk + 1][c] = rb[h].y;
+                Bs[buf][lk + 2][c] = rb[h].z; Bs[buf][lk + 3][c] = rb[h].w;
+            }
         }
     };
-    load(0);
+    load(0, 0);
     store(0);
+    if constexpr (WT) asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
     int cur = 0;
     for (int k0 = 0; k0 < K; k0 += BK) {
         const bool more = k0 + BK < K;
-        if (more) load(k0 + BK);
+        if (more) load(k0 + BK, cur ^ 1);
 #pragma unroll
         for (int kk = 0; kk < BK; ++kk) {
             const float4 a0 = *reinterpret_cast<const float4*>(&As[cur][kk][ty * 4]);
@@ -148,6 +164,7 @@ __global__ __launch_bounds__(256, 2) void k_sgemm(const float* __restrict__ A1, 
         if (more) {
             // the other buffer was last read before the previous barrier
             store(cur ^ 1);
+            if constexpr (WT) asm volatile("cp.async.wait_all;" ::: "memory");
             __syncthreads();
             cur ^= 1;
         }
@@ -161,13 +178,22 @@ __global__ __launch_bounds__(256, 2) void k_sgemm(const float* __restrict__ A1, 
             const int col = n0 + h * 64 + tx * 4;
             float4 v;
             const float2* ar = acc[i >> 1];
-            v.x = ((i & 1) ? ar[h * 4 + 0].y : ar[h * 4 + 0].x) + bias[col + 0];
-            v.y = ((i & 1) ? ar[h * 4 + 1].y : ar[h * 4 + 1].x) + bias[col + 1];
-            v.z = ((i & 1) ? ar[h * 4 + 2].y : ar[h * 4 + 2].x) + bias[col + 2];
-            v.w = ((i & 1) ? ar[h * 4 + 3].y : ar[h * 4 + 3].x) + bias[col + 3];
+            v.x = (i & 1) ? ar[h * 4 + 0].y : ar[h * 4 + 0].x;
+            v.y = (i & 1) ? ar[h * 4 + 1].y : ar[h * 4 + 1].x;
+            v.z = (i & 1) ? ar[h * 4 + 2].y : ar[h * 4 + 2].x;
+            v.w = (i & 1) ? ar[h * 4 + 3].y : ar[h * 4 + 3].x;
+            if constexpr (!WT) {
+                v.x += bias[col + 0]; v.y += bias[col + 1];
+                v.z += bias[col + 2]; v.w += bias[col + 3];
+            }
             if (RELU) {
                 v.x = fmaxf(v.x, 0.f); v.y = fmaxf(v.y, 0.f);
                 v.z = fmaxf(v.z, 0.f); v.w = fmaxf(v.w, 0.f);
+            }
+            if (WT && mask) {
+                const float4 h4 = *reinterpret_cast<const float4*>(mask + (size_t)row * ldc + col);
+                v.x = h4.x > 0.f ? v.x : 0.f; v.y = h4.y > 0.f ? v.y : 0.f;
+                v.z = h4.z > 0.f ? v.z : 0.f; v.w = h4.w > 0.f ? v.w : 0.f;
             }
             *reinterpret_cast<float4*>(C + (size_t)row * ldc + col) = v;
         }
@@ -267,11 +293,19 @@ static cudaError_t gemm(const float* A1, int lda1, int K1, const float* A2, int 
     dim3 grid((M + 127) / 128, L.n / 128);
     note_launch();
     if (relu)
-        k_sgemm<true><<<grid, 256, 0, s>>>(A1, lda1, K1, A2, lda2, K2, a2_off, a2_div, L.W, L.b, C,
-                                           ldc, M, rows_dev, r0);
+        k_sgemm<true, false><<<grid, 256, 0, s>>>(A1, lda1, K1, A2, lda2, K2, a2_off, a2_div, L.W, 0,
+                                                  L.b, nullptr, C, ldc, M, rows_dev, r0);
     else
-        k_sgemm<false><<<grid, 256, 0, s>>>(A1, lda1, K1, A2, lda2, K2, a2_off, a2_div, L.W, L.b, C,
-                                            ldc, M, rows_dev, r0);
+        k_sgemm<false, false><<<grid, 256, 0, s>>>(A1, lda1, K1, A2, lda2, K2, a2_off, a2_div, L.W, 0,
+                                                   L.b, nullptr, C, ldc, M, rows_dev, r0);
+    return cudaGetLastError();
+}
+
+cudaError_t fp32_gemm_back(const float* dY, int n_out, const float* W, int ldw, const float* mask,
+                           float* dX, int M, cudaStream_t s) {
+    note_launch();
+    k_sgemm<false, true><<<dim3((M + 127) / 128, kWidth / 128), 256, 0, s>>>(
+        dY, kWidth, n_out, nullptr, 0, 0, 0, 1, W, ldw, nullptr, mask, dX, kWidth, M, nullptr, 0);
     return cudaGetLastError();
 }
 

@@ -703,42 +703,34 @@ static cudaError_t prop_loss_grad_batch(mcl_map* m, const float* O, const float*
     return cudaGetLastError();
 }
 
-static int alloc_batch(PropBatch& b, long rows) {
-    int rc;
+static void add_batch(Scratch& sc, PropBatch& b, long rows) {
     const long nblk = (rows + kWgChunk - 1) / kWgChunk;
-    if ((rc = cuda_check(cudaMalloc(&b.part, sizeof(float) * nblk * kPN), "batch partials"))) return rc;
-    if ((rc = cuda_check(cudaMalloc(&b.g, sizeof(float) * rows * kPInPad), "batch g"))) return rc;
-    if ((rc = cuda_check(cudaMalloc(&b.h, sizeof(float) * rows * kPDepth * kPW), "batch h"))) return rc;
-    if ((rc = cuda_check(cudaMalloc(&b.da, sizeof(float) * rows * kPDepth * kPW), "batch da"))) return rc;
-    if ((rc = cuda_check(cudaMalloc(&b.s, sizeof(float) * rows), "batch s"))) return rc;
-    return cuda_check(cudaMalloc(&b.ds, sizeof(float) * rows), "batch ds");
-}
-
-static void free_batch(PropBatch& b) {
-    if (b.part) cudaFree(b.part);
-    if (b.g) cudaFree(b.g);
-    if (b.h) cudaFree(b.h);
-    if (b.da) cudaFree(b.da);
-    if (b.s) cudaFree(b.s);
-    if (b.ds) cudaFree(b.ds);
-    b = PropBatch{};
+    sc.add(&b.part, sizeof(float) * nblk * kPN);
+    sc.add(&b.g, sizeof(float) * rows * kPInPad);
+    sc.add(&b.h, sizeof(float) * rows * kPDepth * kPW);
+    sc.add(&b.da, sizeof(float) * rows * kPDepth * kPW);
+    sc.add(&b.s, sizeof(float) * rows);
+    sc.add(&b.ds, sizeof(float) * rows);
 }
 
 int proposal_loss_grad(mcl_map* m, const float* O, const float* D, int n, int nb, float near_z,
                        float far_z, const float* hist, double* d_loss, float* d_grad,
                        cudaStream_t s) {
     PropBatch b{};
-    int rc = alloc_batch(b, (long)n * nb);
-    if (!rc) rc = cuda_check(cudaMemsetAsync(d_loss, 0, sizeof(double), s), "clear loss");
+    Scratch sc;
+    add_batch(sc, b, (long)n * nb);
+    int rc = sc.take(m);
+    if (rc) return rc;
+    rc = cuda_check(cudaMemsetAsync(d_loss, 0, sizeof(double), s), "clear loss");
     if (!rc)
         rc = cuda_check(prop_loss_grad_batch(m, O, D, n, nb, near_z, far_z, hist, 1.0f / n, 1.0 / n, b, d_loss, s),
                         "proposal loss/grad");
     if (!rc)
         rc = cuda_check(cudaMemcpyAsync(d_grad, m->prop_g, sizeof(float) * kPN, cudaMemcpyDeviceToDevice, s),
                         "copy grad");
-    if (!rc) rc = cuda_check(cudaStreamSynchronize(s), "proposal sync");
-    free_batch(b);
-    return rc;
+    // (also after an error: the scratch may be freed or used again)
+    const int rs = cuda_check(cudaStreamSynchronize(s), "proposal sync");
+    return rc ? rc : rs;
 }
 
 int proposal_train(mcl_map* m, const float* d_poses, int n_poses, const int32_t* d_pixels, int B,
@@ -754,29 +746,17 @@ int proposal_train(mcl_map* m, const float* d_poses, int n_poses, const int32_t*
     double* loss_acc = nullptr;
     PropBatch b{};
     const int batch = cfg.batch_rays;
-    auto cleanup = [&]() {
-        if (O) cudaFree(O);
-        if (D) cudaFree(D);
-        if (hist) cudaFree(hist);
-        if (Ob) cudaFree(Ob);
-        if (Db) cudaFree(Db);
-        if (Hb) cudaFree(Hb);
-        if (perm_d) cudaFree(perm_d);
-        if (loss_acc) cudaFree(loss_acc);
-        free_batch(b);
-    };
-    if ((rc = cuda_check(cudaMalloc(&O, sizeof(float) * 3 * n_rays), "train O")) ||
-        (rc = cuda_check(cudaMalloc(&D, sizeof(float) * 3 * n_rays), "train D")) ||
-        (rc = cuda_check(cudaMalloc(&hist, sizeof(float) * nb * n_rays), "train hist")) ||
-        (rc = cuda_check(cudaMalloc(&Ob, sizeof(float) * 3 * batch), "batch O")) ||
-        (rc = cuda_check(cudaMalloc(&Db, sizeof(float) * 3 * batch), "batch D")) ||
-        (rc = cuda_check(cudaMalloc(&Hb, sizeof(float) * nb * batch), "batch hist")) ||
-        (rc = cuda_check(cudaMalloc(&perm_d, sizeof(int) * n_rays), "perm")) ||
-        (rc = cuda_check(cudaMalloc(&loss_acc, sizeof(double)), "loss")) ||
-        (rc = alloc_batch(b, (long)batch * nb))) {
-        cleanup();
-        return rc;
-    }
+    Scratch sc;
+    sc.add(&O, sizeof(float) * 3 * n_rays);
+    sc.add(&D, sizeof(float) * 3 * n_rays);
+    sc.add(&hist, sizeof(float) * nb * n_rays);
+    sc.add(&Ob, sizeof(float) * 3 * batch);
+    sc.add(&Db, sizeof(float) * 3 * batch);
+    sc.add(&Hb, sizeof(float) * nb * batch);
+    sc.add(&perm_d, sizeof(int) * n_rays);
+    sc.add(&loss_acc, sizeof(double));
+    add_batch(sc, b, (long)batch * nb);
+    if ((rc = sc.take(m))) return rc;
     // 1) targets from the full sampler, in chunks of poses that fit the workspace
     const int chunk_poses = std::max(1, std::min(n_poses, m->cfg.max_rays / B));
     for (int p0 = 0; p0 < n_poses && !rc; p0 += chunk_poses) {
@@ -846,8 +826,8 @@ int proposal_train(mcl_map* m, const float* d_poses, int n_poses, const int32_t*
     }
     m->prop_step = step;
     if (!rc) rc = cuda_check(prop_tc_pack(m, s), "pack proposal");
-    if (!rc) rc = cuda_check(cudaStreamSynchronize(s), "train sync");
-    cleanup();
+    const int rs = cuda_check(cudaStreamSynchronize(s), "train sync");
+    if (!rc) rc = rs;
     if (!rc) m->has_proposal = true;
     return rc;
 }
