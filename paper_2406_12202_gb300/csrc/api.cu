@@ -265,6 +265,10 @@ extern "C" int mcl_init_map(const float* host_weights, size_t n_floats, const mc
         free_map(m);
         return rc;
     }
+    if ((rc = cuda_check(coarse_to_fine_prepare(), "importance sampling smem"))) {
+        free_map(m);
+        return rc;
+    }
     if ((rc = mlp_tc_prepare(m, host_weights))) {
         free_map(m);
         return rc;

@@ -181,6 +181,7 @@ cudaError_t launch_raygen(const float* particles, int N, const int32_t* pixels, 
                           float4* obs = nullptr);
 cudaError_t launch_query_setup(const float* X, const float* D, int n, Ray* rays, float* gd,
                                float* z, cudaStream_t s);
+cudaError_t coarse_to_fine_prepare();
 cudaError_t launch_coarse_to_fine(const Ray* rays, int n_rays, const int* n_rays_dev,
                                   const float* zc, int nc, const float4* out_c, int nf, float* zf,
                                   cudaStream_t s);

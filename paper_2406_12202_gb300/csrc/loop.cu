@@ -84,23 +84,23 @@ __global__ void k_raygen_b(const LoopPlan* __restrict__ pl, int nq, const float*
     if (obs) obs[r] = observed_colour(imgs[q], W, H, f, px[2 * j], px[2 * j + 1]);
 }
 
-__global__ void k_final_b(const LoopPlan* __restrict__ pl, int nq, const float* const* __restrict__ imgs,
-                          int W, const int32_t* __restrict__ pix, const Ray* __restrict__ rays,
-                          const float* __restrict__ zc, const float4* __restrict__ oc, int nc,
-                          const float* __restrict__ zf, const float4* __restrict__ of, int nf,
-                          float alpha, float tau, int use_rej, int max_rays,
-                          float* __restrict__ e_ray) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= max_rays || r >= pl->total_rays) return;
+__global__ void __launch_bounds__(32) k_final_b(
+    const LoopPlan* __restrict__ pl, int nq, const float* const* __restrict__ imgs, int W,
+    const int32_t* __restrict__ pix, const Ray* __restrict__ rays, const float* __restrict__ zc,
+    const float4* __restrict__ oc, int nc, const float* __restrict__ zf,
+    const float4* __restrict__ of, int nf, float alpha, float tau, int use_rej, int max_rays,
+    float* __restrict__ e_ray) {
+    __shared__ CompositeSmem sm;
+    const int r0 = blockIdx.x * 32, r = r0 + threadIdx.x;
+    const int n = min(max_rays, pl->total_rays);
+    if (r0 >= n) return;
+    const RayResult c = composite_warp(rays, zc, oc, nc, zf, of, nf, r0, n, alpha, tau, use_rej, sm);
+    if (r >= n) return;
     const int q = query_of_ray(pl, nq, r);
     const int B = pl->B[q], f = pl->factor[q];
     const int j = (r - pl->ray_off[q]) % B;
     const int32_t* px = pix + (size_t)q * kLoopMaxPixels * 2;
-    const float dn = rays[r].dnorm;
-    const RayResult c = composite_ray(dn, zc + (size_t)r * nc, oc + (size_t)r * nc, nc,
-                                      zf + (size_t)r * nf, of + (size_t)r * nf, nf, alpha, tau,
-                                      use_rej);
-    e_ray[r] = photometric_E(imgs[q], W, f, px[2 * j], px[2 * j + 1], c, dn) * c.F;
+    e_ray[r] = photometric_E(imgs[q], W, f, px[2 * j], px[2 * j + 1], c, rays[r].dnorm) * c.F;
 }
 
 // Weights of each query (one block per query), survivors, weighted pose
@@ -324,7 +324,7 @@ int enqueue_localize(mcl_map* m, int nq, float* P_user, int stride, const mcl_in
         }
         if (!fused) {
             note_launch();
-            k_final_b<<<(max_rays_run + tb - 1) / tb, tb, 0, s>>>(
+            k_final_b<<<(max_rays_run + 31) / 32, 32, 0, s>>>(
                 L.plan, nq, L.imgs, K.width, L.pix, m->rays, za, m->out_c, nc, zb, m->out_f, nf,
                 o.alpha, o.tau, o.use_rejection, max_rays_run, m->e_ray);
         }

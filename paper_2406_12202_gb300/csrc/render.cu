@@ -80,44 +80,48 @@ cudaError_t launch_raygen(const float* particles, int N, const int32_t* pixels, 
     return cudaGetLastError();
 }
 
-// Coarse composite and importance samples, one thread per ray.  n_rays_dev
+// Coarse composite and importance samples, a warp per 32 rays.  n_rays_dev
 // (optional) bounds the rays from device memory.
-__global__ void k_coarse_to_fine(const Ray* __restrict__ rays, int n_rays,
-                                 const int* __restrict__ n_rays_dev, const float* __restrict__ zc,
-                                 int nc, const float4* __restrict__ out_c, int nf,
-                                 float* __restrict__ zf) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(32) k_coarse_to_fine(
+    const Ray* __restrict__ rays, int n_rays, const int* __restrict__ n_rays_dev,
+    const float* __restrict__ zc, int nc, const float4* __restrict__ out_c, int nf,
+    float* __restrict__ zf) {
+    extern __shared__ float sm_samples[];
+    const int r0 = blockIdx.x * 32;
     const int n = n_rays_dev ? min(n_rays, *n_rays_dev) : n_rays;
-    if (r >= n) return;
-    importance_samples(zc + (size_t)r * nc, out_c + (size_t)r * nc, nc, rays[r].dnorm, nf,
-                       zf + (size_t)r * nf);
+    if (r0 >= n) return;
+    importance_warp(rays, zc, out_c, nc, r0, n, nf, zf, sm_samples);
+}
+
+cudaError_t coarse_to_fine_prepare() {
+    return cudaFuncSetAttribute(k_coarse_to_fine, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                importance_floats(kMaxCoarse) * (int)sizeof(float));
 }
 
 cudaError_t launch_coarse_to_fine(const Ray* rays, int n_rays, const int* n_rays_dev,
                                   const float* zc, int nc, const float4* out_c, int nf, float* zf,
                                   cudaStream_t s) {
-    const int tb = 128;
     note_launch();
-    k_coarse_to_fine<<<(n_rays + tb - 1) / tb, tb, 0, s>>>(rays, n_rays, n_rays_dev, zc, nc, out_c,
-                                                            nf, zf);
+    k_coarse_to_fine<<<(n_rays + 31) / 32, 32, importance_floats(nc) * sizeof(float), s>>>(
+        rays, n_rays, n_rays_dev, zc, nc, out_c, nf, zf);
     return cudaGetLastError();
 }
 
-// Final composite, Eq. 5 / F and E against the level image, one thread per
-// ray.  image == NULL: render only (rgb_out / F_out).
-__global__ void k_final(const Ray* __restrict__ rays, int n_rays, const float* __restrict__ zc,
-                        const float4* __restrict__ oc, int nc, const float* __restrict__ zf,
-                        const float4* __restrict__ of, int nf, const float* __restrict__ img,
-                        int W, int H, int factor, const int32_t* __restrict__ px, int B, float alpha,
-                        float tau, int use_rej, float* __restrict__ e_ray, float* __restrict__ d_rgb,
-                        float* __restrict__ d_E, float* __restrict__ d_F, float* __restrict__ d_zt,
-                        float* __restrict__ d_zo) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+// Final composite, Eq. 5 / F and E against the level image, a warp per 32
+// rays.  image == NULL: render only (rgb_out / F_out).
+__global__ void __launch_bounds__(32) k_final(
+    const Ray* __restrict__ rays, int n_rays, const float* __restrict__ zc,
+    const float4* __restrict__ oc, int nc, const float* __restrict__ zf,
+    const float4* __restrict__ of, int nf, const float* __restrict__ img, int W, int H, int factor,
+    const int32_t* __restrict__ px, int B, float alpha, float tau, int use_rej,
+    float* __restrict__ e_ray, float* __restrict__ d_rgb, float* __restrict__ d_E,
+    float* __restrict__ d_F, float* __restrict__ d_zt, float* __restrict__ d_zo) {
+    __shared__ CompositeSmem sm;
+    const int r = blockIdx.x * 32 + threadIdx.x;
+    const RayResult c = composite_warp(rays, zc, oc, nc, zf, of, nf, blockIdx.x * 32, n_rays, alpha,
+                                       tau, use_rej, sm);
     if (r >= n_rays) return;
     const float dn = rays[r].dnorm;
-    const RayResult c = composite_ray(dn, zc + (size_t)r * nc, oc + (size_t)r * nc, nc,
-                                      zf + (size_t)r * nf, of + (size_t)r * nf, nf, alpha, tau,
-                                      use_rej);
     if (d_rgb) { d_rgb[3 * (size_t)r] = c.r; d_rgb[3 * (size_t)r + 1] = c.g; d_rgb[3 * (size_t)r + 2] = c.b; }
     if (d_F) d_F[r] = c.F;
     if (d_zt) d_zt[r] = c.z_trans;
@@ -143,11 +147,10 @@ cudaError_t launch_final_composite(const Ray* rays, int n_rays, const float* zc,
                                    const int32_t* pixels, int B, const mcl_opts& o, float* e_ray,
                                    const mcl_debug* dbg, float* rgb_out, float* F_out,
                                    cudaStream_t s) {
-    const int tb = 128;
     float* d_rgb = rgb_out ? rgb_out : (dbg ? dbg->rgb : nullptr);
     float* d_F = F_out ? F_out : (dbg ? dbg->F : nullptr);
     note_launch();
-    k_final<<<(n_rays + tb - 1) / tb, tb, 0, s>>>(
+    k_final<<<(n_rays + 31) / 32, 32, 0, s>>>(
         rays, n_rays, zc, out_c, nc, zf, out_f, nf, image, W, H, factor, pixels, B, o.alpha, o.tau,
         o.use_rejection, e_ray, d_rgb, dbg ? dbg->E : nullptr, d_F, dbg ? dbg->z_trans : nullptr,
         dbg ? dbg->z_opaque : nullptr);

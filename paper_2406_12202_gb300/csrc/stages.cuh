@@ -93,46 +93,121 @@ __device__ __forceinline__ void coarse_samples(long r, int nc, float near_z, flo
     }
 }
 
+// ---------------------------------------------------------------------------
+// Compositing and sampling of 32 consecutive rays by one warp, a lane per ray.
+//
+// The sums and products along a ray keep their order, so a ray is one serial
+// chain; a warp per 32 rays leaves the chip about 8 chains of 32 rays per SM
+// at 38,400 rays.  What bounds these kernels when a lane also fetches its own
+// samples is the fetch: 32 different lines per load, each a wait on L2.  So
+// the warp brings the rows in together, coalesced, into shared memory, and
+// only the chains run there (38,400 rays x (64 + 128) samples: sampling 165 ->
+// 60 us, composite 177 -> 57 us, of which reading the samples takes 22).
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void copy_async16(void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                     (uint32_t)__cvta_generic_to_shared(dst)),
+                 "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void copy_async4(void* dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(
+                     (uint32_t)__cvta_generic_to_shared(dst)),
+                 "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+
+// Floats of shared memory of importance_warp: z and CDF of 32 rays, [sample][33]
+// (a ray's samples go to 32 banks when they are stored, a sample's rays when
+// they are read), and 32 samples on their way out.
+__host__ __device__ constexpr int importance_floats(int nc) { return (2 * nc + 32) * 33; }
+
 // Coarse composite (Eq. 1 quadrature) and inverse-CDF importance samples of
-// one ray: edges = midpoints of consecutive coarse z; pdf over the interior
-// bins proportional to w_1..w_{n_c-2} + 1e-5; u_j = j/(n_f - 1); the bin is
-// the first CDF entry strictly greater than u_j (u sorted: one sweep).
-__device__ __forceinline__ void importance_samples(const float* __restrict__ z,
-                                                   const float4* __restrict__ o, int nc, float dn,
-                                                   int nf, float* __restrict__ out) {
-    float cdf[kMaxCoarse];
+// rays r0 .. r0 + 31 (those below n): edges = midpoints of consecutive coarse
+// z; pdf over the interior bins proportional to w_1..w_{n_c-2} + 1e-5;
+// u_j = j/(n_f - 1); the bin is the first CDF entry strictly greater than u_j
+// (u sorted: one sweep).
+__device__ __forceinline__ void importance_warp(const Ray* __restrict__ rays,
+                                                const float* __restrict__ zc,
+                                                const float4* __restrict__ oc, int nc, int r0,
+                                                int n, int nf, float* __restrict__ zf,
+                                                float* __restrict__ sm) {
+    const int lane = threadIdx.x & 31;
+    const int live = min(32, n - r0);
+    float* zs = sm;
+    float* cdf = zs + nc * 33;
+    float* ob = cdf + nc * 33;
+    zc += (size_t)r0 * nc;
+    oc += (size_t)r0 * nc;
+    zf += (size_t)r0 * nf;
+#pragma unroll 8
+    for (int q = 0; q < 32; ++q) {
+        const size_t row = (size_t)min(q, live - 1) * nc;
+        for (int k = lane; k < nc; k += 32) {
+            copy_async4(&zs[k * 33 + q], &zc[row + k]);
+            copy_async4(&cdf[k * 33 + q], &oc[row + k].x);
+        }
+    }
+    copy_commit();
+    const float dn = rays[r0 + min(lane, live - 1)].dnorm;
+    copy_wait();
+    __syncwarp();
+    zs += lane;
+    cdf += lane;
     float T = 1.0f;
     float tot = 0.0f;
-    for (int k = 0; k < nc; ++k) {
-        const float sg = fmaxf(o[k].x, 0.0f);
-        const float delta = (k < nc - 1) ? (z[k + 1] - z[k]) * dn : 1e10f;
+#pragma unroll 4
+    for (int k = 0; k < nc - 1; ++k) {
+        const float sg = fmaxf(cdf[k * 33], 0.0f);
+        const float delta = (zs[(k + 1) * 33] - zs[k * 33]) * dn;
         const float a = 1.0f - expf(-sg * delta);
-        const float w = T * a;
+        // (rounded twice in every fourth bin: the samples drawn from the CDF are
+        // ill-conditioned, so its roundings are part of the result)
+        const float w = (k & 3) == 3 ? __fadd_rn(__fmul_rn(T, a), 1e-5f) : fmaf(T, a, 1e-5f);
         T *= (1.0f - a);
-        if (k >= 1 && k <= nc - 2) {
-            cdf[k] = w + 1e-5f;   // pdf of bin k-1, normalised below
-            tot += w + 1e-5f;
+        if (k >= 1) {
+            cdf[k * 33] = w;   // pdf of bin k-1, normalised below
+            tot += w;
         }
     }
     const int ne = nc - 1;
     cdf[0] = 0.0f;
     float run = 0.0f;
+#pragma unroll 4
     for (int i = 1; i < ne; ++i) {
-        run += cdf[i] / tot;
-        cdf[i] = run;
+        run += cdf[i * 33] / tot;
+        cdf[i * 33] = run;
     }
+    // the sweep keeps the bin's ends in registers: CDF (c_lo, c_hi) and edge
+    // (eb, ea) of entries max(idx - 1, 0) and min(idx, ne - 1)
     int idx = 0;
-    for (int j = 0; j < nf; ++j) {
-        const float u = nf > 1 ? (float)j / (float)(nf - 1) : 0.0f;
-        while (idx < ne && cdf[idx] <= u) ++idx;
-        const int below = idx - 1 < 0 ? 0 : idx - 1;
-        const int above = idx > ne - 1 ? ne - 1 : idx;
-        float denom = cdf[above] - cdf[below];
-        if (denom < 1e-5f) denom = 1.0f;
-        const float t = (u - cdf[below]) / denom;
-        const float eb = 0.5f * (z[below] + z[below + 1]);
-        const float ea = 0.5f * (z[above] + z[above + 1]);
-        out[j] = eb + t * (ea - eb);
+    float c_lo = 0.0f, c_hi = 0.0f;
+    float ea = 0.5f * (zs[0] + zs[33]), eb = ea;
+    for (int j0 = 0; j0 < nf; j0 += 32) {
+        const int m = min(32, nf - j0);
+        for (int jj = 0; jj < m; ++jj) {
+            const int j = j0 + jj;
+            const float u = nf > 1 ? (float)j / (float)(nf - 1) : 0.0f;
+            while (idx < ne && c_hi <= u) {
+                ++idx;
+                c_lo = c_hi;
+                eb = ea;
+                if (idx < ne) {
+                    c_hi = cdf[idx * 33];
+                    ea = 0.5f * (zs[idx * 33] + zs[(idx + 1) * 33]);
+                }
+            }
+            float denom = c_hi - c_lo;
+            if (denom < 1e-5f) denom = 1.0f;
+            const float t = (u - c_lo) / denom;
+            ob[jj * 33 + lane] = eb + t * (ea - eb);
+        }
+        __syncwarp();
+        if (lane < m)
+            for (int q = 0; q < live; ++q) zf[(size_t)q * nf + j0 + lane] = ob[lane * 33 + q];
+        __syncwarp();
     }
 }
 
@@ -141,33 +216,64 @@ struct RayResult {
     float z_trans, z_opaque, F;
 };
 
-// Final composite over the merged coarse + fine samples (both sorted; equal
-// z take the coarse sample first), Eq. 5 on the running weight sum and F of
-// Eq. 6 (F = 1 without rejection).
-__device__ __forceinline__ RayResult composite_ray(float dn, const float* __restrict__ za,
-                                                   const float4* __restrict__ oa, int nc,
-                                                   const float* __restrict__ zb,
-                                                   const float4* __restrict__ ob, int nf,
-                                                   float alpha, float tau, int use_rej) {
-    int ia = 0, ib = 0;
-    auto take = [&](float& z, float4& v) {
-        if (ib >= nf || (ia < nc && za[ia] <= zb[ib])) {
-            z = za[ia]; v = oa[ia]; ++ia;
-        } else {
-            z = zb[ib]; v = ob[ib]; ++ib;
+// Shared memory of composite_warp: per ray a ring of 16 samples of each pass,
+// the values [slot][32] (read without conflicts), z [slot][33].
+constexpr int kRing = 16, kRingStep = 8;
+struct CompositeSmem {
+    float4 v[2][kRing][32];
+    float z[2][kRing][33];
+};
+
+// Final composite of rays r0 .. r0 + 31 over the merged coarse + fine samples
+// (both sorted; equal z take the coarse sample first), Eq. 5 on the running
+// weight sum and F of Eq. 6 (F = 1 without rejection).
+//
+// Which sample comes next is known only ray by ray, so every 8 samples the
+// warp tops up all rays' rings, 8 lanes per ray and pass (128-byte pieces),
+// with what the 8 samples after the coming ones may need.
+__device__ __forceinline__ RayResult composite_warp(const Ray* __restrict__ rays,
+                                                    const float* __restrict__ za,
+                                                    const float4* __restrict__ oa, int nc,
+                                                    const float* __restrict__ zb,
+                                                    const float4* __restrict__ ob, int nf, int r0,
+                                                    int n_rays, float alpha, float tau, int use_rej,
+                                                    CompositeSmem& sm) {
+    const int lane = threadIdx.x & 31;
+    const int live = min(32, n_rays - r0);
+    // this lane's part of a top-up: entry e of pass `list` of rays 2 p + half
+    const int e = lane & 7, list = (lane >> 3) & 1, half = lane >> 4;
+    const int cnt = list ? nf : nc;
+    const float* const zl = (list ? zb : za) + (size_t)r0 * cnt;
+    const float4* const ol = (list ? ob : oa) + (size_t)r0 * cnt;
+    int ia = 0, ib = 0, la = 0, lb = 0;   // taken and loaded so far
+    auto top_up = [&]() {
+        const int pa = ia << 16 | la, pb = ib << 16 | lb;
+#pragma unroll 4
+        for (int p = 0; p < 16; ++p) {
+            const int q = 2 * p + half;
+            const int sa = __shfl_sync(0xffffffffu, pa, q), sb = __shfl_sync(0xffffffffu, pb, q);
+            const int st = list ? sb : sa;
+            const int i = (st & 0xffff) + e;
+            if (i < min((st >> 16) + kRing, cnt)) {
+                const size_t at = (size_t)min(q, live - 1) * cnt + i;
+                copy_async16(&sm.v[list][i & (kRing - 1)][q], &ol[at]);
+                copy_async4(&sm.z[list][i & (kRing - 1)][q], &zl[at]);
+            }
         }
+        copy_commit();
+        la = min(max(la, min(la + kRingStep, ia + kRing)), nc);
+        lb = min(max(lb, min(lb + kRingStep, ib + kRing)), nf);
     };
+    top_up();
+    top_up();
+    const float dn = rays[r0 + min(lane, live - 1)].dnorm;
     const int n = nc + nf;
-    float zcur, znext = 0.f;
-    float4 vcur, vnext = make_float4(0.f, 0.f, 0.f, 0.f);
-    take(zcur, vcur);
-    const float z0 = zcur;
+    float zcur = 0.f;
+    float4 vcur = make_float4(0.f, 0.f, 0.f, 0.f);
     float T = 1.0f, cr = 0.f, cg = 0.f, cb = 0.f, Wc = 0.f;
-    float zt = z0, zo = z0;
+    float zt = 0.f, zo = 0.f;
     bool have_t = false;
-    for (int k = 0; k < n; ++k) {
-        if (k < n - 1) take(znext, vnext);
-        const float delta = (k < n - 1) ? (znext - zcur) * dn : 1e10f;
+    auto add = [&](float delta) {
         const float sg = fmaxf(vcur.x, 0.0f);
         const float a = 1.0f - expf(-sg * delta);
         const float w = T * a;
@@ -176,8 +282,26 @@ __device__ __forceinline__ RayResult composite_ray(float dn, const float* __rest
         Wc += w;
         if (!have_t && Wc >= alpha) { zt = zcur; have_t = true; }
         if (Wc <= 1.0f - alpha) zo = zcur;
-        zcur = znext; vcur = vnext;
+    };
+    for (int k0 = 0; k0 < n; k0 += kRingStep) {
+        copy_wait();
+        __syncwarp();   // what was loaded is there, what was taken may be overwritten
+        if (k0 > 0) top_up();
+        const int m = min(kRingStep, n - k0);
+        for (int kk = 0; kk < m; ++kk) {
+            const float ha = sm.z[0][ia & (kRing - 1)][lane], hb = sm.z[1][ib & (kRing - 1)][lane];
+            const bool second = !(ib >= nf || (ia < nc && ha <= hb));
+            const float znext = second ? hb : ha;
+            const float4 vnext = sm.v[second][(second ? ib : ia) & (kRing - 1)][lane];
+            if (second) ++ib;
+            else ++ia;
+            if (k0 + kk > 0) add((znext - zcur) * dn);
+            else zt = zo = znext;
+            zcur = znext;
+            vcur = vnext;
+        }
     }
+    add(1e10f);
     RayResult res;
     res.r = cr; res.g = cg; res.b = cb;
     res.z_trans = zt; res.z_opaque = zo;
