@@ -53,35 +53,42 @@ __global__ void k_plan(LoopPlan* __restrict__ pl, const LoopQuery* __restrict__ 
 }
 
 // Pixel set of each query (Floyd's algorithm on SplitMix64, as
-// mcl_draw_pixels): one thread per query.
-__global__ void k_pixels(const LoopPlan* __restrict__ pl, int nq, int W, int H, uint64_t seed,
-                         int t, int32_t* __restrict__ pix) {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= nq) return;
+// mcl_draw_pixels): one warp per query.
+__global__ void __launch_bounds__(32) k_pixels(const LoopPlan* __restrict__ pl, int W, int H,
+                                               uint64_t seed, int t, int32_t* __restrict__ pix) {
+    __shared__ long sm[2][kLoopMaxPixels];
+    const int q = blockIdx.x;
     const int f = pl->factor[q];
-    draw_pixel_set(W / f, H / f, pl->B[q], seed, loop_ctr(q, t, 0), pix + (size_t)q * kLoopMaxPixels * 2);
+    draw_pixel_set(W / f, H / f, pl->B[q], seed, loop_ctr(q, t, 0),
+                   pix + (size_t)q * kLoopMaxPixels * 2, sm[0], sm[1]);
 }
 
-__global__ void k_raygen_b(const LoopPlan* __restrict__ pl, int nq, const float* __restrict__ P,
-                           int stride, const int32_t* __restrict__ pix, float fx, float fy,
-                           float cx, float cy, int nc, float near_z, float far_z, int jitter,
-                           uint64_t seed, int t, int max_rays, Ray* __restrict__ rays,
-                           float* __restrict__ gd, float* __restrict__ zc,
-                           const float* const* __restrict__ imgs, int W, int H,
-                           float4* __restrict__ obs) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= max_rays || r >= pl->total_rays) return;
-    const int q = query_of_ray(pl, nq, r);
-    const int B = pl->B[q], f = pl->factor[q];
+__global__ void __launch_bounds__(32) k_raygen_b(
+    const LoopPlan* __restrict__ pl, int nq, const float* __restrict__ P, int stride,
+    const int32_t* __restrict__ pix, float fx, float fy, float cx, float cy, int nc, float near_z,
+    float far_z, int jitter, uint64_t seed, int t, int max_rays, Ray* __restrict__ rays,
+    float* __restrict__ gd, float* __restrict__ zc, const float* const* __restrict__ imgs, int W,
+    int H, float4* __restrict__ obs) {
+    __shared__ float g[32][kGdPad + 1];
+    const int r0 = blockIdx.x * 32, r = r0 + threadIdx.x;
+    const int n = min(max_rays, pl->total_rays);
+    const int live = min(32, n - r0);
+    if (live <= 0) return;
+    const int q = query_of_ray(pl, nq, min(r, n - 1));
     const int rl = r - pl->ray_off[q];
-    const int i = rl / B, j = rl - (rl / B) * B;
-    const int32_t* px = pix + (size_t)q * kLoopMaxPixels * 2;
-    Ray ray;
-    make_ray(P + 12 * ((size_t)q * stride + i), px[2 * j], px[2 * j + 1], fx / f, fy / f, cx / f,
-             cy / f, ray, gd + (size_t)r * kGdPad);
-    rays[r] = ray;
-    coarse_samples(rl, nc, near_z, far_z, jitter, seed, loop_ctr(q, t, 3), zc + (size_t)r * nc);
-    if (obs) obs[r] = observed_colour(imgs[q], W, H, f, px[2 * j], px[2 * j + 1]);
+    if (r < n) {
+        const int B = pl->B[q], f = pl->factor[q];
+        const int i = rl / B, j = rl - (rl / B) * B;
+        const int32_t* px = pix + (size_t)q * kLoopMaxPixels * 2;
+        Ray ray;
+        make_ray(P + 12 * ((size_t)q * stride + i), px[2 * j], px[2 * j + 1], fx / f, fy / f,
+                 cx / f, cy / f, ray, g[threadIdx.x]);
+        rays[r] = ray;
+        if (obs) obs[r] = observed_colour(imgs[q], W, H, f, px[2 * j], px[2 * j + 1]);
+    }
+    coarse_samples_warp(rl, loop_ctr(q, t, 3), live, nc, near_z, far_z, jitter, seed,
+                        zc + (size_t)r0 * nc);
+    store_gd_warp(g, live, gd + (size_t)r0 * kGdPad);
 }
 
 __global__ void __launch_bounds__(32) k_final_b(
@@ -103,51 +110,47 @@ __global__ void __launch_bounds__(32) k_final_b(
     e_ray[r] = photometric_E(imgs[q], W, f, px[2 * j], px[2 * j + 1], c, rays[r].dnorm) * c.F;
 }
 
-// Weights of each query (one block per query), survivors, weighted pose
+// Weights of each query (one team of CTAs per query), survivors, weighted pose
 // estimate and weighted position spread; one log record per query.
-__global__ __launch_bounds__(kLoopThreads) void k_weights_b(
+__global__ __launch_bounds__(kTeamThreads) void k_weights_b(
     const LoopPlan* __restrict__ pl, LoopQuery* __restrict__ qs, const float* __restrict__ P,
     int stride, const float* __restrict__ e_ray, double s_min, double rho,
     double* __restrict__ l64, double* __restrict__ w, uint8_t* __restrict__ mask,
     mcl_iter_record* __restrict__ log, int iterations, int t, mcl_schedule sch) {
-    const int q = blockIdx.x;
+    __shared__ TeamSmem sm;
+    __shared__ double sh[7][32], m[6], var_sum[1];
+    const Team tm = make_team();
+    const int q = blockIdx.x / tm.ctas;
     const int N = pl->N[q], B = pl->B[q];
     const size_t base = (size_t)q * stride;
-    const int nbad = weights_block(e_ray + pl->ray_off[q], N, B, s_min, rho, nullptr, l64 + base,
-                                   w + base, mask + base, nullptr);
-    __shared__ double sh[32];
-    double m[6];
+    const int nbad = weights_team(tm, sm, e_ray + pl->ray_off[q], N, B, s_min, rho, nullptr,
+                                  l64 + base, w + base, mask + base, nullptr);
     // survivors, weighted mean position, weighted yaw direction
-    double acc_s = 0.0;
-    double am[3] = {0.0, 0.0, 0.0}, ys = 0.0, yc = 0.0;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
+    double acc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    for (int i = tm.first; i < N; i += tm.step) {
         const float* p = P + 12 * (base + i);
         const double wi = w[base + i];
-        acc_s += mask[base + i] ? 1.0 : 0.0;
+        acc[0] += mask[base + i] ? 1.0 : 0.0;
         if (wi > 0.0) {
-            am[0] += wi * p[3]; am[1] += wi * p[7]; am[2] += wi * p[11];
+            acc[1] += wi * p[3]; acc[2] += wi * p[7]; acc[3] += wi * p[11];
             const double yaw = atan2((double)p[2], (double)p[0]);
-            ys += wi * sin(yaw);
-            yc += wi * cos(yaw);
+            acc[4] += wi * sin(yaw);
+            acc[5] += wi * cos(yaw);
         }
     }
-    m[0] = block_sum_d(acc_s, sh);
-    m[1] = block_sum_d(am[0], sh);
-    m[2] = block_sum_d(am[1], sh);
-    m[3] = block_sum_d(am[2], sh);
-    m[4] = block_sum_d(ys, sh);
-    m[5] = block_sum_d(yc, sh);
-    double var = 0.0;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
+    team_sum<6>(tm, N, acc, sh, m);
+    double var[1] = {0.0};
+    for (int i = tm.first; i < N; i += tm.step) {
         const float* p = P + 12 * (base + i);
         const double wi = w[base + i];
         if (wi > 0.0) {
             const double d0 = p[3] - m[1], d1 = p[7] - m[2], d2 = p[11] - m[3];
-            var += wi * (d0 * d0 + d1 * d1 + d2 * d2);
+            var[0] += wi * (d0 * d0 + d1 * d1 + d2 * d2);
         }
     }
-    var = block_sum_d(var, sh);
-    if (threadIdx.x == 0) {
+    team_sum<1>(tm, N, var, sh + 6, var_sum);
+    if (tm.rank == 0 && threadIdx.x == 0) {
+        const double var = var_sum[0];
         qs[q].n_surv = (int)m[0];
         qs[q].wspread = var;
         if (nbad > 0) qs[q].nonfinite += nbad;
@@ -199,24 +202,22 @@ __global__ __launch_bounds__(kLoopThreads) void k_resample_b(
     resample_block(w + base, pl->N[q], pl->Nnext[q], u0, idx + base, cdf + base);
 }
 
-__global__ void k_predict_b(const LoopPlan* __restrict__ pl, int nq, int stride,
-                            const float* __restrict__ Pin, const int32_t* __restrict__ idx,
-                            float sigma_t, float sigma_yaw, uint64_t seed, int t,
-                            float* __restrict__ Pout) {
-    const long g = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= (long)nq * stride) return;
-    const int q = (int)(g / stride), k = (int)(g - (long)q * stride);
-    if (k >= pl->Nnext[q]) return;
+__global__ void __launch_bounds__(128) k_predict_b(
+    const LoopPlan* __restrict__ pl, int nq, int stride, const float* __restrict__ Pin,
+    const int32_t* __restrict__ idx, float sigma_t, float sigma_yaw, uint64_t seed, int t,
+    float* __restrict__ Pout) {
+    const long g = (long)blockIdx.x * 32 + (threadIdx.x >> 2);   // four lanes per particle
+    const int q = min((int)(g / stride), nq - 1), k = (int)(g - (long)q * stride);
+    const bool in = k < stride && k < pl->Nnext[q];
+    if (!__any_sync(0xffffffffu, in)) return;
     const size_t base = (size_t)q * stride;
-    const int src = idx[base + k];
+    const int src = in ? idx[base + k] : -1;
+    const bool ok = src >= 0 && src < pl->N[q];
     float* O = Pout + 12 * (base + k);
-    if (src < 0 || src >= pl->N[q]) {
-        for (int c = 0; c < 12; ++c) O[c] = __int_as_float(0x7fc00000);
-        return;
-    }
-    double qn[4];
-    motion_noise(seed, loop_ctr(q, t, 2), k, sigma_t, sigma_yaw, qn);
-    predict_pose(Pin + 12 * (base + src), qn, O);
+    predict_quad(Pin + 12 * (base + (ok ? src : 0)), seed, loop_ctr(q, t, 2), k, sigma_t, sigma_yaw,
+                 ok, O, nullptr);
+    if (in && !ok)
+        for (int c = threadIdx.x & 3; c < 12; c += 4) O[c] = __int_as_float(0x7fc00000);
 }
 
 __global__ void k_loop_init(LoopQuery* __restrict__ qs, const int* __restrict__ n0, int nq) {
@@ -233,15 +234,16 @@ __global__ void k_loop_final(const LoopQuery* __restrict__ qs, int nq, int* __re
     if (q < nq) n_out[q] = qs[q].N;
 }
 
-__global__ void k_draw_pixels(int W, int H, int B, uint64_t seed, uint64_t ctr,
-                              int32_t* __restrict__ out) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) draw_pixel_set(W, H, B, seed, ctr, out);
+__global__ void __launch_bounds__(32) k_draw_pixels(int W, int H, int B, uint64_t seed,
+                                                    uint64_t ctr, int32_t* __restrict__ out) {
+    extern __shared__ long sm_draws[];
+    draw_pixel_set(W, H, B, seed, ctr, out, sm_draws, sm_draws + B);
 }
 
 cudaError_t launch_draw_pixels(int W, int H, int B, uint64_t seed, uint64_t ctr, int32_t* out,
                                cudaStream_t s) {
     note_launch();
-    k_draw_pixels<<<1, 32, 0, s>>>(W, H, B, seed, ctr, out);
+    k_draw_pixels<<<1, 32, 2 * (size_t)B * sizeof(long), s>>>(W, H, B, seed, ctr, out);
     return cudaGetLastError();
 }
 
@@ -260,7 +262,6 @@ int enqueue_localize(mcl_map* m, int nq, float* P_user, int stride, const mcl_in
     const int nc = prop ? o.n_guided : o.n_coarse, nf = o.n_fine;
     float* const za = prop ? m->zf : m->zc;
     float* const zb = prop ? m->zc : m->zf;
-    const int tb = 128;
     // the NeRF MLP of the precision, rows from the plan in device memory;
     // tensor-core forms with the fused ray epilogues where the shapes allow
     const bool fp32 = o.precision == MCL_PREC_FP32;
@@ -293,8 +294,8 @@ int enqueue_localize(mcl_map* m, int nq, float* P_user, int stride, const mcl_in
     for (int t = 0; t < sch.iterations; ++t) {
         note_launch(4);
         k_plan<<<1, 32, 0, s>>>(L.plan, L.qs, nq, sch, nc, nf);
-        k_pixels<<<1, 64, 0, s>>>(L.plan, nq, K.width, K.height, o.seed, t, L.pix);
-        k_raygen_b<<<(max_rays_run + tb - 1) / tb, tb, 0, s>>>(
+        k_pixels<<<nq, 32, 0, s>>>(L.plan, K.width, K.height, o.seed, t, L.pix);
+        k_raygen_b<<<(max_rays_run + 31) / 32, 32, 0, s>>>(
             L.plan, nq, Pc, stride, L.pix, K.fx, K.fy, K.cx, K.cy, np, o.near_z, o.far_z,
             prop ? 0 : o.jitter, o.seed, t, max_rays_run, m->rays, m->gd, m->zc, L.imgs, K.width,
             K.height, fused ? m->obs : nullptr);
@@ -329,12 +330,14 @@ int enqueue_localize(mcl_map* m, int nq, float* P_user, int stride, const mcl_in
                 o.alpha, o.tau, o.use_rejection, max_rays_run, m->e_ray);
         }
         note_launch(4);
-        k_weights_b<<<nq, kLoopThreads, 0, s>>>(L.plan, L.qs, Pc, stride, m->e_ray, o.s_min,
-                                                 o.rho_reject, m->logw64, L.w, L.mask, d_log,
-                                                 sch.iterations, t, sch);
+        if ((rc = cuda_check(launch_teams(k_weights_b, nq, kTeamMost, s, L.plan, L.qs, Pc, stride,
+                                          m->e_ray, (double)o.s_min, (double)o.rho_reject, m->logw64,
+                                          L.w, L.mask, d_log, sch.iterations, t, sch),
+                             "loop weights")))
+            return rc;
         k_schedule_b<<<1, 64, 0, s>>>(L.plan, L.qs, nq, sch, stride);
         k_resample_b<<<nq, kLoopThreads, 0, s>>>(L.plan, stride, L.w, L.idx, m->cdf, o.seed, t);
-        k_predict_b<<<(unsigned)(((long)nq * stride + tb - 1) / tb), tb, 0, s>>>(
+        k_predict_b<<<(unsigned)(((long)nq * stride + 31) / 32), 128, 0, s>>>(
             L.plan, nq, stride, Pc, L.idx, sch.sigma_t, sch.sigma_yaw, o.seed, t, Pn);
         float* tmp = Pc;
         Pc = Pn;

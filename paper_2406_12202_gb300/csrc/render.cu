@@ -9,23 +9,28 @@
 
 namespace mcl {
 
-// One thread per ray r = i*B + j: pixel-centre ray of particle i through
-// pixel j with the level intrinsics, gamma(d), stratified coarse samples.
-__global__ void k_raygen(const float* __restrict__ P, int N, const int32_t* __restrict__ px,
-                         int B, float fx, float fy, float cx, float cy, int nc, float near_z,
-                         float far_z, int jitter, uint64_t seed, uint64_t ctr,
-                         Ray* __restrict__ rays, float* __restrict__ gd, float* __restrict__ zc,
-                         const float* __restrict__ img, int W, int H, int factor,
-                         float4* __restrict__ obs) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= N * B) return;
-    const int i = r / B, j = r - (r / B) * B;
-    Ray ray;
-    make_ray(P + 12 * (size_t)i, px[2 * j], px[2 * j + 1], fx, fy, cx, cy, ray,
-             gd + (size_t)r * kGdPad);
-    rays[r] = ray;
-    coarse_samples(r, nc, near_z, far_z, jitter, seed, ctr, zc + (size_t)r * nc);
-    if (obs) obs[r] = observed_colour(img, W, H, factor, px[2 * j], px[2 * j + 1]);
+// Ray r = i*B + j: pixel-centre ray of particle i through pixel j with the level
+// intrinsics, gamma(d), stratified coarse samples.  One warp per block and a
+// lane per ray for the FP64 part (five divisions, a root; about two FP64 lanes
+// per SM), so that a small step's rays spread over the SMs; samples and gamma(d)
+// go out coalesced (38,400 rays x 64 samples: 27 -> 21 us).
+__global__ void __launch_bounds__(32) k_raygen(
+    const float* __restrict__ P, int N, const int32_t* __restrict__ px, int B, float fx, float fy,
+    float cx, float cy, int nc, float near_z, float far_z, int jitter, uint64_t seed, uint64_t ctr,
+    Ray* __restrict__ rays, float* __restrict__ gd, float* __restrict__ zc,
+    const float* __restrict__ img, int W, int H, int factor, float4* __restrict__ obs) {
+    __shared__ float g[32][kGdPad + 1];
+    const int r0 = blockIdx.x * 32, r = r0 + threadIdx.x;
+    const int live = min(32, N * B - r0);
+    if (r < N * B) {
+        const int i = r / B, j = r - (r / B) * B;
+        Ray ray;
+        make_ray(P + 12 * (size_t)i, px[2 * j], px[2 * j + 1], fx, fy, cx, cy, ray, g[threadIdx.x]);
+        rays[r] = ray;
+        if (obs) obs[r] = observed_colour(img, W, H, factor, px[2 * j], px[2 * j + 1]);
+    }
+    coarse_samples_warp(r, ctr, live, nc, near_z, far_z, jitter, seed, zc + (size_t)r0 * nc);
+    store_gd_warp(g, live, gd + (size_t)r0 * kGdPad);
 }
 
 // Point queries: one "ray" per point with o = x, d = 0 and one sample at
@@ -71,9 +76,8 @@ cudaError_t launch_raygen(const float* particles, int N, const int32_t* pixels, 
                           float fy, float cx, float cy, const mcl_opts& o, Ray* rays, float* gd,
                           float* zc, cudaStream_t s, const float* image, int W, int H, int factor,
                           float4* obs) {
-    const int n = N * B, tb = 128;
     note_launch();
-    k_raygen<<<(n + tb - 1) / tb, tb, 0, s>>>(particles, N, pixels, B, fx, fy, cx, cy, o.n_coarse,
+    k_raygen<<<(N * B + 31) / 32, 32, 0, s>>>(particles, N, pixels, B, fx, fy, cx, cy, o.n_coarse,
                                                o.near_z, o.far_z, o.jitter, o.seed, o.counter,
                                                rays, gd, zc, image, W, H, factor,
                                                image ? obs : nullptr);
@@ -157,14 +161,14 @@ cudaError_t launch_final_composite(const Ray* rays, int n_rays, const float* zc,
     return cudaGetLastError();
 }
 
-constexpr int kNormThreads = 1024;
-
-__global__ __launch_bounds__(kNormThreads) void k_weights(
+__global__ __launch_bounds__(kTeamThreads) void k_weights(
     const float* __restrict__ e_ray, int N, int B, double s_min, double rho,
     float* __restrict__ logw, double* __restrict__ l64, double* __restrict__ w,
     uint8_t* __restrict__ mask, float* __restrict__ S_dbg, Status* status) {
-    const int nbad = weights_block(e_ray, N, B, s_min, rho, logw, l64, w, mask, S_dbg);
-    if (threadIdx.x == 0 && nbad > 0) {
+    __shared__ TeamSmem sm;
+    const Team t = make_team();
+    const int nbad = weights_team(t, sm, e_ray, N, B, s_min, rho, logw, l64, w, mask, S_dbg);
+    if (t.rank == 0 && threadIdx.x == 0 && nbad > 0) {
         atomicAdd(&status->n_nonfinite, nbad);
         atomicCAS(&status->code, 0, MCL_ERR_NONFINITE);
     }
@@ -174,9 +178,8 @@ cudaError_t launch_weights(const float* e_ray, int N, int B, const mcl_opts& o, 
                            double* logw64, double* w, uint8_t* mask, float* S_dbg, Status* status,
                            cudaStream_t s) {
     note_launch();
-    k_weights<<<1, kNormThreads, 0, s>>>(e_ray, N, B, o.s_min, o.rho_reject, logw, logw64, w, mask,
-                                         S_dbg, status);
-    return cudaGetLastError();
+    return launch_teams(k_weights, 1, team_ctas(N), s, e_ray, N, B, (double)o.s_min,
+                       (double)o.rho_reject, logw, logw64, w, mask, S_dbg, status);
 }
 
 }  // namespace mcl

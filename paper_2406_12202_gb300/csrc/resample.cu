@@ -20,33 +20,36 @@ __global__ __launch_bounds__(kResThreads) void k_resample(const double* __restri
 cudaError_t launch_resample(const double* w, int n_in, int n_out, double u0, int32_t* idx,
                             unsigned long long* cdf, Status* status, cudaStream_t s) {
     note_launch();
-    k_resample<<<1, kResThreads, 0, s>>>(w, n_in, n_out, u0, idx, cdf, status);
+    // no more warps than there are weights or indices: idle ones would still
+    // take part in the FP64 maximum and the scan
+    const int most = n_in > n_out ? n_in : n_out;
+    const int tb = most < kResThreads ? (most + 31) / 32 * 32 : kResThreads;
+    k_resample<<<1, tb, 0, s>>>(w, n_in, n_out, u0, idx, cdf, status);
     return cudaGetLastError();
 }
 
-// Prediction: out_k = in_{idx_k} * Exp(rho, (0, yaw, 0)) (stages.cuh).
-__global__ void k_predict(const float* __restrict__ in, int n_in, const int32_t* __restrict__ idx,
-                          int n, const float* __restrict__ odom, float sigma_t, float sigma_yaw,
-                          uint64_t seed, uint64_t ctr, float* __restrict__ out) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
-    const int src = idx ? idx[k] : k;
+// Prediction: out_k = in_{idx_k} * Exp(rho, (0, yaw, 0)) (stages.cuh), four
+// lanes per particle and one warp per block (small sets spread over the SMs).
+__global__ void __launch_bounds__(32) k_predict(const float* __restrict__ in, int n_in,
+                                                const int32_t* __restrict__ idx, int n,
+                                                const float* __restrict__ odom, float sigma_t,
+                                                float sigma_yaw, uint64_t seed, uint64_t ctr,
+                                                float* __restrict__ out) {
+    const int k = blockIdx.x * 8 + (threadIdx.x >> 2);
+    const int src = k < n ? (idx ? idx[k] : k) : -1;
+    const bool ok = src >= 0 && src < n_in;
     float* O = out + 12 * (size_t)k;
-    if (src < 0 || src >= n_in) {
-        for (int c = 0; c < 12; ++c) O[c] = __int_as_float(0x7fc00000);
-        return;
-    }
-    double q[4];
-    motion_noise(seed, ctr, k, sigma_t, sigma_yaw, q);
-    predict_pose(in + 12 * (size_t)src, q, O, odom);
+    predict_quad(in + (ok ? 12 * (size_t)src : 0), seed, ctr, k, sigma_t, sigma_yaw, ok, O, odom);
+    if (k < n && !ok)
+        for (int c = threadIdx.x & 3; c < 12; c += 4) O[c] = __int_as_float(0x7fc00000);
 }
 
 cudaError_t launch_predict(const float* in, int n_in, const int32_t* idx, int n_out,
                            const float* odom, float sigma_t, float sigma_yaw, uint64_t seed,
                            uint64_t counter, float* out, cudaStream_t s) {
     note_launch();
-    k_predict<<<(n_out + 127) / 128, 128, 0, s>>>(in, n_in, idx, n_out, odom, sigma_t, sigma_yaw, seed,
-                                                   counter, out);
+    k_predict<<<(n_out + 7) / 8, 32, 0, s>>>(in, n_in, idx, n_out, odom, sigma_t, sigma_yaw, seed,
+                                             counter, out);
     return cudaGetLastError();
 }
 

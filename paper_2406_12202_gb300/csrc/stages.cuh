@@ -5,6 +5,8 @@
 #pragma once
 #include <math.h>
 
+#include <utility>
+
 #include "internal.cuh"
 #include "rng.cuh"
 
@@ -65,32 +67,61 @@ __device__ __forceinline__ void make_ray(const float* __restrict__ p, int u, int
 // for j = n-B .. n-1 draw t uniform in [0, j] and take t unless already
 // taken, else j.  t = floor(r (j + 1) / 2^64), r = value j-(n-B) of
 // SplitMix64 stream (seed, ctr).  out[2i], out[2i+1] = (q % W, q / W).
-// One thread; O(B^2) membership tests.
+// One warp: the draws are independent, the tests against the pixels taken so
+// far go 32 at a time.  t and c: B values of scratch each.
 __device__ __forceinline__ void draw_pixel_set(int W, int H, int B, uint64_t seed, uint64_t ctr,
-                                               int32_t* __restrict__ out) {
-    const long n = (long)W * H;
-    for (long j = n - B, m = 0; j < n; ++j, ++m) {
-        const uint64_t r = cb_rand(seed, ctr, (uint64_t)(j - (n - B)));
-        const long t = (long)(((u128)r * (u128)(uint64_t)(j + 1)) >> 64);
+                                               int32_t* __restrict__ out, long* __restrict__ t,
+                                               long* __restrict__ c) {
+    const int lane = threadIdx.x & 31;
+    const long j0 = (long)W * H - B;
+    for (int m = lane; m < B; m += 32) {
+        const uint64_t r = cb_rand(seed, ctr, (uint64_t)m);
+        t[m] = (long)(((u128)r * (u128)(uint64_t)(j0 + m + 1)) >> 64);
+    }
+    __syncwarp();
+    for (int m = 0; m < B; ++m) {
+        const long tm = t[m];
         bool dup = false;
-        for (long i = 0; i < m; ++i)
-            if ((long)out[2 * i + 1] * W + out[2 * i] == t) { dup = true; break; }
-        const long c = dup ? j : t;
-        out[2 * m] = (int32_t)(c % W);
-        out[2 * m + 1] = (int32_t)(c / W);
+        for (int i = lane; i < m; i += 32) dup = dup || c[i] == tm;
+        dup = __any_sync(0xffffffffu, dup);
+        if (lane == 0) c[m] = dup ? j0 + m : tm;
+        __syncwarp();
+    }
+    for (int m = lane; m < B; m += 32) {
+        out[2 * m] = (int32_t)(c[m] % W);
+        out[2 * m + 1] = (int32_t)(c[m] / W);
     }
 }
 
-// Stratified coarse samples of ray r: z_k = near + (far - near)(k + u_k)/n_c,
-// u_k = 1/2 or value r*n_c + k of SplitMix64 stream (seed, ctr).
-__device__ __forceinline__ void coarse_samples(long r, int nc, float near_z, float far_z,
-                                               int jitter, uint64_t seed, uint64_t ctr,
-                                               float* __restrict__ z) {
+// Stratified coarse samples of the warp's rays r0 .. r0 + live - 1, ray index r
+// of its stream and counter ctr per lane: z_k = near + (far - near)(k + u_k)/n_c,
+// u_k = 1/2 or value r*n_c + k of SplitMix64 stream (seed, ctr).  A lane per
+// sample, so that a ray's samples go out together.  The 53 bits of u_k are
+// rounded to FP32 once, as the FP64 value k 2^-53 would be.
+__device__ __forceinline__ void coarse_samples_warp(long r, uint64_t ctr, int live, int nc,
+                                                    float near_z, float far_z, int jitter,
+                                                    uint64_t seed, float* __restrict__ z) {
+    const int lane = threadIdx.x & 31;
     const float span = far_z - near_z;
-    for (int k = 0; k < nc; ++k) {
-        const float uk = jitter ? (float)cb_uniform(seed, ctr, (uint64_t)r * nc + k) : 0.5f;
-        z[k] = near_z + span * ((float)k + uk) / (float)nc;
+    const int total = live * nc;
+#pragma unroll 4
+    for (int e0 = 0; e0 < total; e0 += 32) {
+        const int e = e0 + lane;
+        const int q = e / nc, k = e - q * nc;   // (q mod 32 in the last, partial turn)
+        const uint64_t at = (uint64_t)__shfl_sync(0xffffffffu, (long long)r, q) * nc + k;
+        const uint64_t c = __shfl_sync(0xffffffffu, (unsigned long long)ctr, q);
+        const float uk = jitter ? (float)(cb_rand(seed, c, at) >> 11) * 0x1.0p-53f : 0.5f;
+        if (e < total) z[e] = near_z + span * ((float)k + uk) / (float)nc;
     }
+}
+
+// Store the warp's gamma(d) rows (lane's row in g[lane][..]) coalesced.
+__device__ __forceinline__ void store_gd_warp(const float (&g)[32][kGdPad + 1], int live,
+                                              float* __restrict__ gd) {
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+#pragma unroll 8
+    for (int q = 0; q < live; ++q) gd[(size_t)q * kGdPad + lane] = g[q][lane];
 }
 
 // ---------------------------------------------------------------------------
@@ -406,25 +437,127 @@ __device__ __forceinline__ u64 block_scan_u64(u64 v, u64* sh, u64* total) {
 }
 
 // ---------------------------------------------------------------------------
-// Eq. 6 weights of one particle set, by one block: S_i = sum_j E_ij F_ij
-// (FP32, j order), log w_i = 4 (log B - log max(S_i, s_min)), normalisation
-// w_i = exp(log w_i - logsumexp) in FP64, mask_i = (w_i >= rho / N).
-// Non-finite S_i -> log w = -inf (returned count of such particles).
+// Eq. 6 weights of one particle set, by one cluster of C CTAs of 128 threads
+// (C = 1, 2, 4, 8): S_i = sum_j E_ij F_ij (FP32, j order), log w_i = 4 (log B -
+// log max(S_i, s_min)), normalisation w_i = exp(log w_i - logsumexp) in FP64,
+// mask_i = (w_i >= rho / N).  Non-finite S_i -> log w = -inf (returned count of
+// such particles).
+//
+// FP64 is what this costs: the chip has about two FP64 lanes per SM, so a
+// function over 32 warps is 32 times its time over one.  Hence the cluster
+// (a particle's functions run on eight SMs at once), and everything that is
+// the same for all particles is evaluated by one warp.  The particles fall to
+// the threads as to one block of 1,024 (particle i to thread i mod 1,024,
+// whose warps go round the CTAs), and the sums over them are taken over its
+// 32 warps in that order, so the figures do not depend on C.  32 particles x 8
+// pixels: 26 us by one block, 10 now; 600 x 64: 54 and 13.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ int weights_block(const float* __restrict__ e_ray, int N, int B,
-                                             double s_min, double rho, float* __restrict__ logw,
-                                             double* __restrict__ l64, double* __restrict__ w,
-                                             uint8_t* __restrict__ mask, float* __restrict__ S_dbg) {
-    __shared__ double sh[32];
-    __shared__ int nbad;
-    if (threadIdx.x == 0) nbad = 0;
+constexpr int kTeamThreads = 128, kTeamMost = 8;
+// CTAs for n particles: all eight unless fewer warps hold one particle a lane
+inline int team_ctas(int n) { return n <= 32 ? 1 : n <= 64 ? 2 : n <= 128 ? 4 : kTeamMost; }
+
+struct Team {
+    int rank, ctas;      // this CTA of how many
+    int warp, lane;      // warp of the whole team
+    int first, step;     // particles first, first + step, ...
+};
+__device__ __forceinline__ Team make_team() {
+    Team t;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(t.rank));
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(t.ctas));
+    t.lane = threadIdx.x & 31;
+    t.warp = (threadIdx.x >> 5) * t.ctas + t.rank;
+    t.first = t.warp * 32 + t.lane;
+    t.step = t.ctas * kTeamThreads;
+    return t;
+}
+__device__ __forceinline__ void team_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::
+                     : "memory");
+}
+// v to the same variable of every CTA of the team, by the first lanes of a warp
+__device__ __forceinline__ void team_store(const Team& t, double* at, double v) {
+    if (t.lane < t.ctas) {
+        uint32_t a;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+                     : "=r"(a)
+                     : "r"((uint32_t)__cvta_generic_to_shared(at)), "r"(t.lane));
+        asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+    }
+}
+__device__ __forceinline__ double warp_sum_d(double v) {
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+__device__ __forceinline__ double warp_max_d(double v) {
+    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
+}
+// Sums over the team of K values per thread (warps without a particle hold
+// zeros and skip their part); sh: K rows of 32, res: K, both shared memory.
+// Ends with the results in res in every CTA.
+template <int K>
+__device__ __forceinline__ void team_sum(const Team& t, int n, const double (&v)[K],
+                                         double (*sh)[32], double* res) {
+    const bool live = t.warp * 32 < n;
+#pragma unroll
+    for (int k = 0; k < K; ++k) team_store(t, &sh[k][t.warp], live ? warp_sum_d(v[k]) : 0.0);
+    team_barrier();
+    const int w = threadIdx.x >> 5;
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+        if ((k & 3) == w) {
+            const double s = warp_sum_d(t.lane < t.ctas * 4 ? sh[k][t.lane] : 0.0);
+            if (t.lane == 0) res[k] = s;
+        }
     __syncthreads();
-    const double logB = log((double)B);
-    double mx = -INFINITY;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
+}
+
+// A launch of `teams` teams of `ctas` CTAs.
+template <typename... P, typename... A>
+cudaError_t launch_teams(void (*fn)(P...), int teams, int ctas, cudaStream_t s, A&&... args) {
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3((unsigned)(teams * ctas));
+    c.blockDim = dim3(kTeamThreads);
+    c.stream = s;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)ctas;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, fn, std::forward<A>(args)...);
+}
+
+struct TeamSmem {
+    double log_b, lse, mx;
+    double max_sh[32], sum_sh[1][32], sum[1];
+    double bad_sh[1][32], bad[1];
+};
+
+__device__ __forceinline__ int weights_team(const Team& t, TeamSmem& sm,
+                                            const float* __restrict__ e_ray, int N, int B,
+                                            double s_min, double rho, float* __restrict__ logw,
+                                            double* __restrict__ l64, double* __restrict__ w,
+                                            uint8_t* __restrict__ mask,
+                                            float* __restrict__ S_dbg) {
+    const int wid = threadIdx.x >> 5;
+    if (wid == 3 && t.lane == 0) sm.log_b = log((double)B);
+    // S of the first particle while the fourth warp takes the logarithm
+    auto total = [&](int i) {
         const float* e = e_ray + (size_t)i * B;
         float S = 0.0f;
+#pragma unroll 16
         for (int j = 0; j < B; ++j) S += e[j];
+        return S;
+    };
+    float S = t.first < N ? total(t.first) : 0.0f;
+    team_barrier();   // also: every CTA of the team runs before one stores into another
+    const double logB = sm.log_b;
+    double mx = -INFINITY;
+    int nbad = 0;
+    for (int i = t.first; i < N; i += t.step) {
+        if (i != t.first) S = total(i);
         if (S_dbg) S_dbg[i] = S;
         double l;
         if (isfinite(S)) {
@@ -432,26 +565,42 @@ __device__ __forceinline__ int weights_block(const float* __restrict__ e_ray, in
             l = 4.0 * (logB - log(sc));
         } else {
             l = -INFINITY;
-            atomicAdd(&nbad, 1);
+            ++nbad;
         }
         l64[i] = l;
         if (logw) logw[i] = (float)l;
         mx = fmax(mx, l);
     }
-    mx = block_max_d(mx, sh);
-    double acc = 0.0;
+    // (log w may be NaN only through s_min; fmax passes it by)
+    const bool live = t.warp * 32 < N;
+    nbad = __reduce_add_sync(0xffffffffu, nbad);
+    team_store(t, &sm.max_sh[t.warp], live ? warp_max_d(mx) : -INFINITY);
+    team_store(t, &sm.bad_sh[0][t.warp], (double)nbad);
+    team_barrier();
+    mx = t.lane < t.ctas * 4 ? sm.max_sh[t.lane] : -INFINITY;
+    if (wid == 0) {
+        mx = warp_max_d(mx);
+        if (t.lane == 0) sm.mx = mx;
+    } else if (wid == 1) {
+        nbad = __reduce_add_sync(0xffffffffu, t.lane < t.ctas * 4 ? (int)sm.bad_sh[0][t.lane] : 0);
+        if (t.lane == 0) sm.bad[0] = (double)nbad;
+    }
+    __syncthreads();
+    mx = sm.mx;
+    double acc[1] = {0.0};
     if (mx > -INFINITY)
-        for (int i = threadIdx.x; i < N; i += blockDim.x) acc += exp(l64[i] - mx);
-    acc = block_sum_d(acc, sh);
-    const double lse = mx + log(acc);
+        for (int i = t.first; i < N; i += t.step) acc[0] += exp(l64[i] - mx);
+    team_sum<1>(t, N, acc, sm.sum_sh, sm.sum);
+    if (wid == 0 && t.lane == 0) sm.lse = mx + log(sm.sum[0]);
     const double thr = rho / (double)N;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
+    __syncthreads();
+    const double lse = sm.lse;
+    for (int i = t.first; i < N; i += t.step) {
         const double wi = (mx > -INFINITY) ? exp(l64[i] - lse) : 0.0;
         w[i] = wi;
         mask[i] = (uint8_t)(wi >= thr && wi > 0.0);
     }
-    __syncthreads();
-    return nbad;
+    return (int)sm.bad[0];
 }
 
 // ---------------------------------------------------------------------------
@@ -517,30 +666,42 @@ __device__ __forceinline__ bool resample_block(const double* __restrict__ w, int
 }
 
 // ---------------------------------------------------------------------------
-// Prediction of one particle: O = P * Exp(q[0..2], (0, q[3], 0)) in FP64.
-// SE(3) exponential: R = I + a K + b K^2, t = (I + b K + c K^2) rho with
-// K = [omega]x, th = |omega|, a = sin th / th, b = (1 - cos th)/th^2,
-// c = (th - sin th)/th^3 (series values below th = 1e-8).
+// Prediction of one particle by four lanes: O = P * Exp(q[0..2], (0, q[3], 0))
+// in FP64 (optionally P * O_t * Exp: odom is the 3x4 relative motion O_t, NULL
+// for the identity).  SE(3) exponential: R = I + a K + b K^2, t = (I + b K + c
+// K^2) rho with K = [omega]x, th = |omega|, a = sin th / th, b = (1 - cos
+// th)/th^2, c = (th - sin th)/th^3 (series values below th = 1e-8).
+//
+// A chain of FP64 functions: its latency is the whole cost of a small call, and
+// the FP64 lanes that of a large one.  Lane c draws normal c of the motion
+// noise (normals 4k .. 4k+3 of stream (seed, ctr), scaled by (sigma_t, sigma_t,
+// sigma_t, sigma_yaw)), lanes 0..2 divide for a, b and c at once, and lane r
+// forms row r of the result (32 particles: 19 us with a lane each, 10 now).  All
+// four lanes enter together; `live` lanes 0..2
+// store.
 // ---------------------------------------------------------------------------
-// x Exp(delta) for the pose P (optionally x O_t Exp(delta): odom is the 3x4
-// relative motion O_t, NULL for the identity), FP64 arithmetic.
-__device__ __forceinline__ void predict_pose(const float* __restrict__ P0, const double q[4],
-                                             float* __restrict__ O,
-                                             const float* __restrict__ odom = nullptr) {
-    double P[12];
+__device__ __forceinline__ void predict_quad(const float* __restrict__ P0, uint64_t seed,
+                                             uint64_t ctr, long k, float sigma_t, float sigma_yaw,
+                                             bool live, float* __restrict__ O,
+                                             const float* __restrict__ odom) {
+    const int c4 = threadIdx.x & 3, base = threadIdx.x & 28, r = min(c4, 2);
+    double q[4];
+    const double mine =
+        (c4 < 3 ? (double)sigma_t : (double)sigma_yaw) * cb_normal(seed, ctr, 4ull * k + c4);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) q[c] = __shfl_sync(0xffffffffu, mine, base + c);
+    double P[4];
     if (odom) {
 #pragma unroll
-        for (int r = 0; r < 3; ++r)
+        for (int c = 0; c < 4; ++c) {
+            double s = (c == 3) ? (double)P0[4 * r + 3] : 0.0;
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                double s = (c == 3) ? (double)P0[4 * r + 3] : 0.0;
-#pragma unroll
-                for (int m = 0; m < 3; ++m) s += (double)P0[4 * r + m] * (double)odom[4 * m + c];
-                P[4 * r + c] = s;
-            }
+            for (int m = 0; m < 3; ++m) s += (double)P0[4 * r + m] * (double)odom[4 * m + c];
+            P[c] = s;
+        }
     } else {
 #pragma unroll
-        for (int k = 0; k < 12; ++k) P[k] = (double)P0[k];
+        for (int c = 0; c < 4; ++c) P[c] = (double)P0[4 * r + c];
     }
     const double om[3] = {0.0, q[3], 0.0};
     const double th2 = om[0] * om[0] + om[1] * om[1] + om[2] * om[2];
@@ -548,48 +709,41 @@ __device__ __forceinline__ void predict_pose(const float* __restrict__ P0, const
     const double K[9] = {0.0, -om[2], om[1], om[2], 0.0, -om[0], -om[1], om[0], 0.0};
     double K2[9];
 #pragma unroll
-    for (int r = 0; r < 3; ++r)
+    for (int i = 0; i < 3; ++i)
 #pragma unroll
         for (int c = 0; c < 3; ++c)
-            K2[3 * r + c] = K[3 * r] * K[c] + K[3 * r + 1] * K[3 + c] + K[3 * r + 2] * K[6 + c];
-    double a, b, cc;
-    if (th < 1e-8) {
-        a = 1.0; b = 0.5; cc = 1.0 / 6.0;
-    } else {
-        a = sin(th) / th;
-        b = (1.0 - cos(th)) / th2;
-        cc = (th - sin(th)) / (th2 * th);
-    }
+            K2[3 * i + c] = K[3 * i] * K[c] + K[3 * i + 1] * K[3 + c] + K[3 * i + 2] * K[6 + c];
+    const double sn = sin(th), cs = cos(th);
+    const double num = r == 0 ? sn : r == 1 ? 1.0 - cs : th - sn;
+    const double den = r == 0 ? th : r == 1 ? th2 : th2 * th;
+    const double abc = th < 1e-8 ? (r == 0 ? 1.0 : r == 1 ? 0.5 : 1.0 / 6.0) : num / den;
+    const double a = __shfl_sync(0xffffffffu, abc, base);
+    const double b = __shfl_sync(0xffffffffu, abc, base + 1);
+    const double cc = __shfl_sync(0xffffffffu, abc, base + 2);
     double E[12];
 #pragma unroll
-    for (int r = 0; r < 3; ++r) {
+    for (int i = 0; i < 3; ++i) {
         double t = 0.0;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            const double I = (r == c) ? 1.0 : 0.0;
-            E[4 * r + c] = I + a * K[3 * r + c] + b * K2[3 * r + c];
-            t += (I + b * K[3 * r + c] + cc * K2[3 * r + c]) * q[c];
+            const double I = (i == c) ? 1.0 : 0.0;
+            E[4 * i + c] = I + a * K[3 * i + c] + b * K2[3 * i + c];
+            t += (I + b * K[3 * i + c] + cc * K2[3 * i + c]) * q[c];
         }
-        E[4 * r + 3] = t;
+        E[4 * i + 3] = t;
     }
+    float v[4];
 #pragma unroll
-    for (int r = 0; r < 3; ++r)
+    for (int c = 0; c < 4; ++c) {
+        double s = (c == 3) ? P[3] : 0.0;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            double s = (c == 3) ? P[4 * r + 3] : 0.0;
+        for (int m = 0; m < 3; ++m) s += P[m] * E[4 * m + c];
+        v[c] = (float)s;
+    }
+    if (live && c4 < 3) {
 #pragma unroll
-            for (int m = 0; m < 3; ++m) s += P[4 * r + m] * E[4 * m + c];
-            O[4 * r + c] = (float)s;
-        }
-}
-
-// Motion noise of particle k: normals 4k .. 4k+3 of stream (seed, ctr)
-// scaled by (sigma_t, sigma_t, sigma_t, sigma_yaw).
-__device__ __forceinline__ void motion_noise(uint64_t seed, uint64_t ctr, long k, float sigma_t,
-                                             float sigma_yaw, double q[4]) {
-#pragma unroll
-    for (int c = 0; c < 4; ++c)
-        q[c] = (c < 3 ? (double)sigma_t : (double)sigma_yaw) * cb_normal(seed, ctr, 4ull * k + c);
+        for (int c = 0; c < 4; ++c) O[4 * r + c] = v[c];
+    }
 }
 
 // Mean position and trace of the population covariance (FP64), one block.
