@@ -7,11 +7,16 @@
 // layers, linear density head) is small enough to stay resident: the four
 // 64 x 64 weight matrices (the first K-padded from 39) live in shared memory
 // as BF16 in the 128-byte-swizzled K-major layout for the whole kernel.
-// Each CTA runs four warpgroups, each owning 128-row tiles, 64 TMEM columns
+// Each CTA runs seven warpgroups, each owning 128-row tiles, 64 TMEM columns
 // and a 16 KB activation tile; per tile and layer one thread of the group
 // issues four 128 x 64 x 16 MMAs, the group reads the accumulators back,
-// applies bias + ReLU and writes the next layer's BF16 operand.  The four
-// groups interleave, so one group's epilogue overlaps the others' MMAs.
+// applies bias + ReLU and writes the next layer's BF16 operand.  The groups
+// interleave, so one group's epilogue overlaps the others' MMAs; a tile is a
+// chain of waits (encoding, then per layer MMA, TMEM load, store), so the
+// groups in flight are what bounds it.  Seven are what 72 registers a thread
+// allow without spills, with the accumulators read 32 columns at a time.  A run
+// of 16 queries (12 updates): 544 ms with four groups, 538 with six, 536 with
+// seven or eight.
 // Every wait is bounded (tc_ptx.cuh).
 #include <math.h>
 
@@ -25,7 +30,7 @@ using namespace tc;
 namespace {
 
 constexpr int kPL = 6, kPIn = 39, kPW = 64;
-constexpr int kGroups = 4;                         // warpgroups (tile slots) per CTA
+constexpr int kGroups = 7;                         // warpgroups (tile slots) per CTA
 constexpr int kThreadsTc = 128 * kGroups;
 constexpr uint32_t kLayerBytes = 64 * 128;         // one 64 x 64 BF16 matrix, 128-byte rows
 constexpr uint32_t kTileBytes = 128 * 128;         // one 128-row activation tile (64 BF16 per row)
@@ -68,6 +73,43 @@ __device__ __forceinline__ void prop_pe_bf16(const float x[3], uint32_t (&pk)[32
     for (int i = 0; i < 32; ++i) pk[i] = pack_bf16x2(v[2 * i], v[2 * i + 1]);
 }
 
+// 32 accumulator columns and their biases -> relu(acc + bias) as 16 BF16
+// pairs: packed FP32 additions, one rounding to BF16, the ReLU on the pairs
+// (the maximum with zero of a rounded value is the rounded maximum).
+__device__ __forceinline__ void relu_bf16(const uint32_t (&v)[32], const float* b, uint32_t* pk) {
+    const float4* b4 = reinterpret_cast<const float4*>(b);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const float4 x = b4[i];
+        const float2 lo = __fadd2_rn(make_float2(__uint_as_float(v[4 * i]), __uint_as_float(v[4 * i + 1])),
+                                     make_float2(x.x, x.y));
+        const float2 hi = __fadd2_rn(make_float2(__uint_as_float(v[4 * i + 2]), __uint_as_float(v[4 * i + 3])),
+                                     make_float2(x.z, x.w));
+        asm("max.bf16x2 %0, %1, %2;" : "=r"(pk[2 * i]) : "r"(pack_bf16x2(lo.x, lo.y)), "r"(0u));
+        asm("max.bf16x2 %0, %1, %2;" : "=r"(pk[2 * i + 1]) : "r"(pack_bf16x2(hi.x, hi.y)), "r"(0u));
+    }
+}
+
+// s + sum relu(acc + bias) w over 32 columns, in column order.
+__device__ __forceinline__ float head_sum(const uint32_t (&v)[32], const float* b, const float* w,
+                                          float s) {
+    const float4* b4 = reinterpret_cast<const float4*>(b);
+    const float4* w4 = reinterpret_cast<const float4*>(w);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const float4 x = b4[i], h = w4[i];
+        const float2 lo = __fadd2_rn(make_float2(__uint_as_float(v[4 * i]), __uint_as_float(v[4 * i + 1])),
+                                     make_float2(x.x, x.y));
+        const float2 hi = __fadd2_rn(make_float2(__uint_as_float(v[4 * i + 2]), __uint_as_float(v[4 * i + 3])),
+                                     make_float2(x.z, x.w));
+        s = fmaf(fmaxf(lo.x, 0.0f), h.x, s);
+        s = fmaf(fmaxf(lo.y, 0.0f), h.y, s);
+        s = fmaf(fmaxf(hi.x, 0.0f), h.z, s);
+        s = fmaf(fmaxf(hi.y, 0.0f), h.w, s);
+    }
+    return s;
+}
+
 }  // namespace
 
 // FP32 blob -> BF16 weight matrices [4][64 rows][64 k] in the 128-byte
@@ -89,7 +131,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
               int* __restrict__ abort_flag, int* __restrict__ status_code) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ PBars bars;
-    __shared__ float s_bias[4 * kPW + kPW + 1];
+    __shared__ __align__(16) float s_bias[4 * kPW + kPW + 1];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const uint32_t s_w = smem_u32(smem);
     const uint32_t s_a = s_w + 4 * kLayerBytes;
@@ -116,7 +158,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
         fence_mbar_init();
     }
     if (warp == 0) {
-        tmem_alloc(smem_u32(&bars.tmem_base), 32 * 2 * kGroups);   // 64 columns per group
+        tmem_alloc(smem_u32(&bars.tmem_base), 512);   // 64 columns per group, a power of two
         tmem_relinquish();
     }
     fence_proxy_async_smem();
@@ -135,14 +177,16 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
     const uint32_t idesc = idesc_bf16(128, 64);
     uint32_t ph_ready = 0, ph_done = 0;
     bool ok = true;
-    for (long long tile = (long long)blockIdx.x * kGroups + grp; tile < n_tiles && ok;
+    for (long long tile = (long long)grp * gridDim.x + blockIdx.x; tile < n_tiles && ok;
          tile += (long long)gridDim.x * kGroups) {
         const long long row = tile * 128 + r;
         const bool valid = row < rows;
         {
             uint32_t pk[32];
             if (valid) {
-                const Ray R = rays[row / n_p];
+                // (a 64-bit quotient is some hundred instructions, so only where needed)
+                const Ray R = rays[rows < 0x80000000ll ? (long long)((uint32_t)row / (uint32_t)n_p)
+                                                       : row / n_p];
                 const float zz = z[row];
                 const float x[3] = {fmaf(zz, R.dx, R.ox), fmaf(zz, R.dy, R.oy), fmaf(zz, R.dz, R.oz)};
                 prop_pe_bf16(x, pk);
@@ -181,37 +225,31 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
             }
             ph_done ^= 1u;
             tc_fence_after();
-            uint32_t va[32], vb[32];
-            tmem_ld32(t_lane, va);
-            tmem_ld32(t_lane + 32, vb);
+            uint32_t v[32];
+            tmem_ld32(t_lane, v);
             tmem_ld_wait();
             const float* b = s_bias + l * kPW;
             if (l < 3) {
-                uint32_t pk[32];
+                uint32_t pk[16];
 #pragma unroll
-                for (int i = 0; i < 16; ++i)
-                    pk[i] = pack_bf16x2(fmaxf(__uint_as_float(va[2 * i]) + b[2 * i], 0.0f),
-                                        fmaxf(__uint_as_float(va[2 * i + 1]) + b[2 * i + 1], 0.0f));
+                for (int h = 0; h < 2; ++h) {
+                    relu_bf16(v, b + 32 * h, pk);
+                    if (h == 0) tmem_ld32(t_lane + 32, v);
 #pragma unroll
-                for (int i = 0; i < 16; ++i)
-                    pk[16 + i] = pack_bf16x2(fmaxf(__uint_as_float(vb[2 * i]) + b[32 + 2 * i], 0.0f),
-                                             fmaxf(__uint_as_float(vb[2 * i + 1]) + b[33 + 2 * i], 0.0f));
-#pragma unroll
-                for (int j = 0; j < 8; ++j)
-                    st_shared_v4(a_tile + sw128_offset(r, j), pk[4 * j], pk[4 * j + 1], pk[4 * j + 2],
-                                 pk[4 * j + 3]);
+                    for (int j = 0; j < 4; ++j)
+                        st_shared_v4(a_tile + sw128_offset(r, 4 * h + j), pk[4 * j], pk[4 * j + 1],
+                                     pk[4 * j + 2], pk[4 * j + 3]);
+                    if (h == 0) tmem_ld_wait();
+                }
                 fence_proxy_async_smem();
                 tc_fence_before();
                 mbar_arrive(bar_ready);
             } else {
                 const float* hw = s_bias + 4 * kPW;
-                float s = hw[kPW];
-#pragma unroll
-                for (int i = 0; i < 32; ++i) s = fmaf(fmaxf(__uint_as_float(va[i]) + b[i], 0.0f), hw[i], s);
-#pragma unroll
-                for (int i = 0; i < 32; ++i)
-                    s = fmaf(fmaxf(__uint_as_float(vb[i]) + b[32 + i], 0.0f), hw[32 + i], s);
-                sigma = s;
+                sigma = head_sum(v, b, hw, hw[kPW]);
+                tmem_ld32(t_lane + 32, v);
+                tmem_ld_wait();
+                sigma = head_sum(v, b + 32, hw + 32, sigma);
                 tc_fence_before();
             }
         }
@@ -227,7 +265,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
     __syncthreads();
     if (warp == 0) {
         tc_fence_after();
-        tmem_dealloc(tmem, 32 * 2 * kGroups);
+        tmem_dealloc(tmem, 512);
     }
 }
 
@@ -245,8 +283,8 @@ cudaError_t launch_prop_infer_tc(mcl_map* m, const Ray* rays, const float* z, in
                                  const int* n_rays_dev, float4* out, int n_sm, cudaStream_t s) {
     const long long rows = (long long)n_rays * n_p;
     const long long tiles = (rows + 127) / 128;
-    long long grid = (tiles + kGroups - 1) / kGroups;
-    if (grid > n_sm) grid = n_sm;
+    // the tiles go to the SMs first and to the groups of each then
+    long long grid = tiles < n_sm ? tiles : n_sm;
     if (grid < 1) grid = 1;
     cudaError_t e = cudaMemsetAsync(m->prop_abort, 0, sizeof(int), s);
     if (e) return e;
