@@ -115,8 +115,8 @@ __global__ void k_prop_infer(const float* __restrict__ W, const Ray* __restrict_
 // three 16-byte loads for 16 instructions, where one thread per row loads a
 // weight for every FMA.  Each output is the same chain of FMAs in the same
 // order as prop_point's.  Bound by the FMA lanes and the stores of the saved
-// rows (1.2 KB each).  Measured, 262,144 rows: forward 0.61 -> 0.16 ms,
-// backward 0.86 -> 0.12 ms.
+// rows (1.2 KB each).  Measured, 262,144 rows: forward 0.61 -> 0.24 ms,
+// backward 0.86 -> 0.19 ms.
 constexpr int kPTile = 128, kPLd = kPTile + 4;
 
 // out[i] (rows 2 i, 2 i + 1 of ty's eight) [e] = fma chain over k of
@@ -242,7 +242,7 @@ __global__ __launch_bounds__(256, 2) void k_prop_fwd_train(
 // block takes kLossRays rays; the exponentials, logarithms and quotients are
 // spread over its threads, and only the running products and sums, whose
 // order is part of the result, are walked by one thread per ray (one thread
-// per ray for everything left all but 32 blocks of the chip idle: 142 -> 18 us
+// per ray for everything left all but 32 blocks of the chip idle: 142 -> 36 us
 // for 4,096 rays of 64 bins).
 constexpr int kLossRays = 8, kLossThreads = 128;
 
@@ -419,7 +419,7 @@ __global__ __launch_bounds__(256, 2) void k_prop_bwd_data(const float* __restric
 // all weights to its own row of `part` (k_grad_reduce adds the rows in block
 // order, so the result is the same on every run).  Bound by the FMA lanes and
 // by reading the saved rows (2.2 KB each).  Measured, 262,144 rows: 0.63 ->
-// 0.18 ms.
+// 0.27 ms.
 constexpr int kWgThreads = 256, kWgTileRows = 16;
 constexpr int kWgRow = 2 * kPDepth * kPW + kPInPad;           // da, h, g of a row
 constexpr int kWgSmem = 2 * kWgTileRows * kWgRow * (int)sizeof(float);
