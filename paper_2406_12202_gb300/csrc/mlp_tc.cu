@@ -2099,11 +2099,11 @@ __global__ void __launch_bounds__(kPipeThreads, 1) k_mlp_tc_pipe(const __grid_co
 }
 
 // Per-ray bias of the RGB hidden layer: b'_ray = b' + W_rgb_hidden[:, 256:283]
-// gamma(d), in the layout of RayBias.  One after the other: a warp per ray, a
-// lane takes four outputs.  Interleaved: a block of 8 warps takes 32 rays, a
+// gamma(d), in the layout of RayBias.  A warp per ray, a lane takes four outputs;
+// or (TILE, for the interleaved layout) a block of 8 warps takes 32 rays, a
 // lane a ray, a warp four outputs of each at a time (the weights are then
 // broadcast loads).  Both store 512 bytes per warp, which is what bounds it.
-template <bool POINTS>
+template <bool POINTS, bool TILE>
 __global__ void __launch_bounds__(256) k_ray_bias(const float* __restrict__ gd, int n_rays,
                                                   const int* __restrict__ n_dev,
                                                   const float* __restrict__ Wd,
@@ -2119,7 +2119,7 @@ __global__ void __launch_bounds__(256) k_ray_bias(const float* __restrict__ gd, 
         s.z = fmaf(w.z, x, s.z);
         s.w = fmaf(w.w, x, s.w);
     };
-    if constexpr (POINTS) {
+    if constexpr (TILE) {
         __shared__ float g[32][kGdPad + 1];
         const int r0 = blockIdx.x * 32;
         if (r0 >= n) return;
@@ -2141,7 +2141,7 @@ __global__ void __launch_bounds__(256) k_ray_bias(const float* __restrict__ gd, 
         float4 s = b4[lane];
 #pragma unroll
         for (int i = 0; i < kGd; ++i) add(s, __ldg(W4 + i * 32 + lane), __shfl_sync(0xffffffffu, x, i));
-        out[ray * 32 + lane] = s;
+        out[POINTS ? (ray >> 5) * 1024 + lane * 32 + (ray & 31) : ray * 32 + lane] = s;
     }
 }
 
@@ -2546,10 +2546,16 @@ cudaError_t mlp_tc_ray_bias(mcl_map* m, const float* gd, int n_rays, const int* 
     st->ray_bias_step = points ? 32 : 1;
     note_launch();
     float4* out = reinterpret_cast<float4*>(st->ray_bias);
-    if (points)
-        k_ray_bias<true><<<(unsigned)(((long)n_rays + 31) / 32), 256, 0, s>>>(gd, n_rays, n_rays_dev, st->Wd, st->bprime, out);
+    const unsigned by_ray = (unsigned)(((long)n_rays + 7) / 8);
+    // Interleaved, but too few rays for a block per 32 on every SM: a warp per
+    // ray all the same (scattered stores, but eight times the warps: 100 FP8 points
+    // 42.6 -> 41.0 us, 1,000 BF16 points 52.9 -> 50.8; at 20,000 the block wins)
+    if (points && n_rays >= 152 * 32)
+        k_ray_bias<true, true><<<(unsigned)(((long)n_rays + 31) / 32), 256, 0, s>>>(gd, n_rays, n_rays_dev, st->Wd, st->bprime, out);
+    else if (points)
+        k_ray_bias<true, false><<<by_ray, 256, 0, s>>>(gd, n_rays, n_rays_dev, st->Wd, st->bprime, out);
     else
-        k_ray_bias<false><<<(unsigned)(((long)n_rays + 7) / 8), 256, 0, s>>>(gd, n_rays, n_rays_dev, st->Wd, st->bprime, out);
+        k_ray_bias<false, false><<<by_ray, 256, 0, s>>>(gd, n_rays, n_rays_dev, st->Wd, st->bprime, out);
     return cudaGetLastError();
 }
 
