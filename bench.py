@@ -36,6 +36,8 @@ WL = dict(workload="full update: 600 particles x 64 px of 400x400, 64+128 sample
           N=600, B=64, W=400, H=400, focal=555.6, n_coarse=64, n_fine=128, level=2,
           sigma_t=0.05, sigma_yaw=0.05, map_seed=0)
 MAC_PER_SAMPLE_FP32 = 593408   # unfused MLP: 8 trunk layers, sigma, feature, rgb head
+MAC_PER_SAMPLE_FOLDED = 524416  # with the feature layer folded into the RGB hidden layer
+MAC_DENSITY_FP32 = 491264      # trunk and density head alone
 METRIC = "MCL update ms and ray-samples/s vs plain FP32 GPU form, at stated pose/RGB error"
 UNIT = "ray-samples/s"
 
@@ -919,16 +921,22 @@ def run_ours(args):
             dist.destroy_process_group()
         return
 
-    # roofline of the dominant kernel of the headline step: the FP32 SIMT
-    # GEMMs of the NeRF MLP (FP32 FMA lanes are the bound)
+    # roofline of the headline step's MLP: every sample as three FP16 products
+    # on the tensor cores, and the densities that importance samples are drawn
+    # from on the FP32 FMA lanes; the peak is the rate at which both would run
+    # at their measured / nominal rates, one after the other
     mlp_ms = (phases["mlp_coarse"] + phases["mlp_fine"]) / args.steps
     mhz = peaks.get("sm_max_mhz", 2070.0)
-    peak = 152 * 128 * 2 * mhz * 1e6 / 1e12
-    roof = {"bound": "alu", "achieved": 2.0 * MAC_PER_SAMPLE_FP32 * rows / (mlp_ms / 1e3) / 1e12,
-            "peak": peak, "unit": "TFLOP/s",
-            "peak_source": f"152 SMs x 128 FP32 lanes x 2 FLOP x {mhz:.0f} MHz ({peak_src} "
-                           "max SM clock)",
-            "kernel": "NeRF MLP, plain FP32 form (k_sgemm layers, PE, heads; coarse + fine)",
+    fma = 152 * 128 * 2 * mhz * 1e6 / 1e12
+    flop = 2.0 * MAC_PER_SAMPLE_FP32 * rows / 1e12
+    first = rows * wl["n_coarse"] / (wl["n_coarse"] + wl["n_fine"])
+    floor_s = (2.0 * MAC_DENSITY_FP32 * first / 1e12 / fma +
+               3 * 2.0 * MAC_PER_SAMPLE_FOLDED * rows / 1e12 / peaks["bf16_tflops"])
+    roof = {"bound": "alu + tensor", "achieved": flop / (mlp_ms / 1e3), "peak": flop / floor_s,
+            "unit": "TFLOP/s",
+            "peak_source": f"first-pass densities at 152 SMs x 128 FP32 lanes x 2 FLOP x {mhz:.0f} "
+                           f"MHz, three FP16 products per sample at bf16_tflops ({peak_src})",
+            "kernel": "NeRF MLP, FP32 form (k_mlp_split; k_sgemm layers for first-pass densities)",
             "mlp_ms_per_step": mlp_ms}
     roof["frac"] = roof["achieved"] / roof["peak"]
     roof["traffic"] = profiled_traffic("k_sgemm_c2_fp32", ("mlp_fp32.cu",))
