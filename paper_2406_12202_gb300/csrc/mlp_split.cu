@@ -39,7 +39,7 @@
 // 64 columns (800) and the hand-over to the even CTA (500).  Measured: 600 x
 // 64 rays of 64 + 128 samples 155.4 -> 15.7 ms by themselves, 58.4 with the
 // first pass's densities from the SIMT kernels (mlp_fp32); 262,144 points
-// 5.62 -> 0.79 ms, 1,000 points 303 -> 66 us.
+// 5.62 -> 0.79 ms, 1,000 points 304 -> 61 us.
 //
 // Warp roles: warp 0 streams the weights; warp 1 issues the MMAs (even CTA)
 // or tells the even CTA that a block has landed (odd CTA); warp 2 (even CTA:
