@@ -42,7 +42,7 @@ struct FitBuf {
     float *m1 = nullptr, *m2 = nullptr;   // Adam moments
 };
 
-int alloc_buf(mcl_map* m, Scratch& sc, FitBuf& b, long B, bool adam) {
+int alloc_buf(mcl_map* m, Scratch& sc, FitBuf& b, long B, bool adam, cudaStream_t s) {
     b.B = B;
     const long nchunk = (B + kWgRows - 1) / kWgRows;
     sc.add(&b.x, sizeof(float) * 3 * B);
@@ -72,8 +72,10 @@ int alloc_buf(mcl_map* m, Scratch& sc, FitBuf& b, long B, bool adam) {
     int rc;
     if ((rc = sc.take(m))) return rc;
     if (adam) {
-        if ((rc = cuda_check(cudaMemset(b.m1, 0, sizeof(float) * m->w32_n), "clear moments")) ||
-            (rc = cuda_check(cudaMemset(b.m2, 0, sizeof(float) * m->w32_n), "clear moments")))
+        // on the run's own stream: the steps on s are not ordered after work of
+        // the default stream, and the block may hold an earlier call's values
+        if ((rc = cuda_check(cudaMemsetAsync(b.m1, 0, sizeof(float) * m->w32_n, s), "clear moments")) ||
+            (rc = cuda_check(cudaMemsetAsync(b.m2, 0, sizeof(float) * m->w32_n, s), "clear moments")))
             return rc;
     }
     return MCL_OK;
@@ -454,7 +456,7 @@ int map_loss_grad(mcl_map* m, const float* d_x, const float* d_dir, const float*
                   float sigma_weight, double* d_loss, float* d_grad, cudaStream_t s) {
     FitBuf b;
     Scratch sc;
-    int rc = alloc_buf(m, sc, b, n, false);
+    int rc = alloc_buf(m, sc, b, n, false, s);
     if (rc) return rc;
     note_launch();
     k_fit_gather<<<(n + 255) / 256, 256, 0, s>>>(d_x, d_dir, d_target, nullptr, 0, n, b.x, b.dir, b.tgt);
@@ -491,7 +493,7 @@ int fit_map(mcl_map* m, const float* d_x, const float* d_dir, const float* d_tar
     int* perm_d = nullptr;
     Scratch sc;
     sc.add(&perm_d, sizeof(int) * n);
-    int rc = alloc_buf(m, sc, b, B, true);
+    int rc = alloc_buf(m, sc, b, B, true, s);
     std::mt19937_64 rng(cfg.seed);
     std::vector<int> perm(n);
     for (int i = 0; i < n; ++i) perm[i] = i;
