@@ -112,6 +112,7 @@ struct __align__(8) SplitBars {
     uint64_t full[kStages], pfull[kStages], empty[kStages];   // pfull: the odd CTA's copy (even CTA)
     uint64_t acc_full[2], acc_empty[2];
     uint64_t a_ready[4], g_ready, g_free, drain, head[4], pair[4];
+    uint64_t ex_ready;           // ex_g of the unit written (within the CTA)
     uint32_t tmem_base;
 };
 
@@ -179,6 +180,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         }
         mbar_init(smem_u32(&bars.g_ready), 2 * 4);
         mbar_init(smem_u32(&bars.g_free), 1);
+        mbar_init(smem_u32(&bars.ex_ready), 4);
         mbar_init(smem_u32(&bars.drain), 1);
         fence_mbar_init();
     }
@@ -251,7 +253,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         put2(62, carry, 0.f);
         fence_proxy_async_smem();
         __syncwarp();
-        if (lane == 0) mbar_arrive_peer(b_g_ready);
+        // gamma(x) is the tensor core's (the even CTA's barrier); ex_g is read
+        // by this CTA's epilogue threads with ordinary loads, and what they
+        // wait for otherwise comes back through the other CTA and the MMAs
+        if (lane == 0) {
+            mbar_arrive(smem_u32(&bars.ex_ready));
+            mbar_arrive_peer(b_g_ready);
+        }
     };
     // registers: launched with 168 per thread (3 warpgroups, 504 shares); the
     // epilogue's two warpgroups take 224 each, the first one keeps 56
@@ -437,6 +445,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         };
         if (u0 < n_units && j == 0) encode(u0, 0, r);
         for (int u = u0; u < n_units && ok; u += du, ++it) {
+            // (written over for unit it + 2 only after the skip layer's MMAs of
+            // unit it + 1, whose operands every warp here has stored after its
+            // last use of unit it's)
+            if (!mbar_wait(smem_u32(&bars.ex_ready), it & 1u, abort_flag)) { ok = false; break; }
             for (int l = 0; l < 8 && ok; ++l) {
                 const int nch = chunks_of(l);
 #pragma unroll

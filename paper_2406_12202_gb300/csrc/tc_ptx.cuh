@@ -159,7 +159,9 @@ __device__ __forceinline__ uint32_t mapa_shared(uint32_t addr, uint32_t rank) {
 // release at CTA scope: the arrivals only tell the even CTA's tensor core of
 // shared-memory writes already made visible by fence.proxy.async, or of TMEM
 // reads that have completed.  (A cluster-scope release waits for every
-// earlier global and local store.)
+// earlier global and local store.)  It does not order ordinary loads and stores
+// of other threads, even those of the arriving CTA: what its own threads read
+// from shared memory has a barrier within the CTA beside it.
 __device__ __forceinline__ void mbar_arrive_peer(uint32_t cluster_addr) {
     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
