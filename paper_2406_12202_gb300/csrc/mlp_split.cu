@@ -602,37 +602,43 @@ struct SplitState {
 };
 
 // Whether the FP16 pairs are as exact as FP32 for the map.  A pair keeps 22 to
-// 23 bits of an operand (0.5 units of FP32's last place, rms), which in a sum
-// of many comparable terms is below the rounding of an FP32 FMA chain, but
-// not in a sum of a few: a row that only copies an input is exact in FP32.
-// The line: (sum |w|)^2 / sum w^2, the number of equal terms that a row's
-// weights are worth, is at least 8 on average over each layer's rows.
-// Measured relative to the largest outputs: He-normal maps (rows worth 40 to
-// 200) 3e-7 to 7e-7 against 4e-7 to 1.3e-6 of the FMA chain, weights falling
-// as 2^-k with the frequency (13 in the first layer) 5e-7 to 7e-7 against
-// 1.0e-6 to 1.3e-6; a hand-set map of copies (1) 2e-5 against 3e-7.  A row
-// below 2^-14 of its layer's largest weight would also lose bits to the
+// 23 bits of an operand, which costs a row's sum about 0.6 units of FP32's last
+// place however many terms it has.  A chain of FMAs rounds once per term, by 0.3
+// units of the sum so far: sqrt(R) times that in all, where R is the sum over the
+// terms of (partial sum / sum)^2, for weights of random sign the partial sums of
+// w^2.  n equal terms make R = n / 2; a row that copies an input, R = 1 and no
+// error at all.  So EVERY row that is not zero has to have an R above the line
+// (a mean over a layer would let rows of copies hide among dense ones).
+// Measured, density error (rms) of the pairs over that of the chain, all layers
+// with k weights of 256 per row (R = k / 2): k = 16 2.7 to 4.3, 33 1.5 to 3.1,
+// 64 1.1 to 1.8, 96 0.9 to 1.5, 128 0.7 to 1.3, 256 (He-normal) 0.5 to 0.8; one
+// such layer among dense ones is 0.5 from k = 16 on.  The first layer's inputs
+// are none of them zero: 16 weights of 63 1.5, 24 0.55.  Dense maps have R of 18
+// at least in the first layer and above 100 in the others.  (Maps fitted to a
+// scene are dense in this sense: density 1.2 to 1.4 in the mean and 0.7 to 0.8 in
+// the largest error, colours 0.4; a hand-set map of copies 70.)
+// A row below 2^-14 of its layer's largest weight would also lose bits to the
 // layer's common scale.
 bool pairs_are_exact(const std::function<double(int, int, int)>& W) {
     for (int l = 0; l < kLayers; ++l) {
         const int rows = l == 8 ? kRgbW + 1 : kWidth, K = l == 0 ? 64 : (l == kSkip ? 320 : 256);
-        double terms = 0.0, layer_max = 0.0, row_min = INFINITY;
-        int used = 0;
+        const double line = l == 0 ? 12.0 : 48.0;
+        double layer_max = 0.0, row_min = INFINITY;
         for (int n = 0; n < rows; ++n) {
-            double s1 = 0.0, s2 = 0.0, mx = 0.0;
-            for (int k = 0; k < K; ++k) {
+            double s2 = 0.0, r = 0.0, mx = 0.0;
+            for (int k = 0; k < K; ++k) {   // in the chain's order
                 const double w = fabs(W(l, n, k));
-                s1 += w;
+                if (!(w > 0.0)) continue;
                 s2 += w * w;
+                r += s2;
                 mx = std::max(mx, w);
             }
             if (!(s2 > 0.0)) continue;
-            ++used;
-            terms += s1 * s1 / s2;
+            if (r < line * s2) return false;
             layer_max = std::max(layer_max, mx);
             row_min = std::min(row_min, mx);
         }
-        if (used && (terms / used < 8.0 || row_min < layer_max * 0x1p-14)) return false;
+        if (row_min < layer_max * 0x1p-14) return false;
     }
     return true;
 }
