@@ -445,11 +445,11 @@ int mcl_autotune(mcl_map* map, int precision, long long rows, int* chosen, float
 
 /* Failure detection test hook (no counterpart in the paper).  The next
  * n_launches launches of the tensor-core NeRF MLP on this map (any entry
- * point that runs it) use the untuned single-CTA kernel of their precision
- * with its weight stream held back and every bounded wait of the kernel
- * limited to wait_ms: the wait for the first weight block runs out, the
- * kernel's warps stop, release their tensor memory and exit, and the map's
- * status word records MCL_ERR_TIMEOUT (mcl_read_status).  The launching call
+ * point that runs it, in FP32 those of maps that run on the tensor cores) use
+ * the untuned kernel of their precision with its weight stream held back and
+ * every bounded wait of the kernel limited to wait_ms: the wait for the first
+ * weight block runs out, the kernel's warps stop, release their tensor memory
+ * and exit, and the map's status word records MCL_ERR_TIMEOUT (mcl_read_status).  The launching call
  * itself returns MCL_OK (the device sees the failure after the call has
  * returned); outputs of the stalled launches are undefined.  Later launches
  * run normally.  No GPU fault, trap or endless wait is involved.

@@ -247,6 +247,8 @@ int mlp_tc_autotune(mcl_map* m, int precision, long long rows, int* chosen, floa
                     cudaStream_t s);
 bool mlp_tc_tuned(const mcl_map* m, int precision);
 int mlp_tc_hold_weights(mcl_map* m, int n_launches, unsigned long long wait_ns);
+// Whether this MLP launch is to be held (and counts it); sets its wait limit.
+bool mlp_tc_take_hold(mcl_map* m, unsigned long long* wait_ns);
 // points: the rays are point queries (one sample each) in `precision`.
 cudaError_t mlp_tc_ray_bias(mcl_map* m, const float* gd, int n_rays, const int* n_rays_dev,
                             cudaStream_t s, bool points = false, int precision = MCL_PREC_FP32);

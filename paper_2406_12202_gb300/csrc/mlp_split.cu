@@ -103,6 +103,8 @@ struct SplitParams {
     float4* out;
     int* abort_flag;
     int* status_code;
+    unsigned long long wait_ns;  // limit of the bounded waits
+    int hold_weights;            // failure-injection hook: no copies are issued
     float cs[kLayers];           // 1 / (weight scale of the layer), see kUnbias
     float b_sigma;
     float b_out[3];
@@ -267,13 +269,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
         if (warp == 0) {
             // ------------------------------------------------ weight stream (both CTAs)
-            if (lane == 0) {
+            if (lane == 0 && !p.hold_weights) {
                 uint32_t g = 0;   // blocks: lo and hi of every chunk
                 for (int u = u0; u < n_units && ok; u += du) {
                     const uint8_t* src = p.wblocks;
                     for (int b = 0; b < 2 * kChunks; ++b, ++g, src += kBlockBytes) {
                         const uint32_t st = g % kStages;
-                        if (!mbar_wait(smem_u32(&bars.empty[st]), ((g / kStages) & 1u) ^ 1u, abort_flag)) {
+                        if (!mbar_wait(smem_u32(&bars.empty[st]), ((g / kStages) & 1u) ^ 1u, abort_flag, p.wait_ns)) {
                             ok = false;
                             break;
                         }
@@ -294,7 +296,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                 for (int u = u0; u < n_units && ok; u += du)
                     for (int b = 0; b < 2 * kChunks; ++b, ++g) {
                         const uint32_t st = g % kStages;
-                        if (!mbar_wait(smem_u32(&bars.full[st]), (g / kStages) & 1u, abort_flag)) {
+                        if (!mbar_wait(smem_u32(&bars.full[st]), (g / kStages) & 1u, abort_flag, p.wait_ns)) {
                             ok = false;
                             break;
                         }
@@ -363,8 +365,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                 uint32_t i = 0, it = 0;
                 auto block = [&](uint32_t g) -> bool {   // block g present in both CTAs
                     const uint32_t st = g % kStages, ph = (g / kStages) & 1u;
-                    return mbar_wait(smem_u32(&bars.full[st]), ph, abort_flag) &&
-                           mbar_wait(smem_u32(&bars.pfull[st]), ph, abort_flag);
+                    return mbar_wait(smem_u32(&bars.full[st]), ph, abort_flag, p.wait_ns) &&
+                           mbar_wait(smem_u32(&bars.pfull[st]), ph, abort_flag, p.wait_ns);
                 };
                 for (int u = u0; u < n_units && ok; u += du, ++it) {
                     for (int l = 0; l < kLayers && ok; ++l) {
@@ -373,9 +375,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                             const int ac = act_chunk(l, c);
                             // what arrives last in the steady state, last
                             bool good = block(2 * i);
-                            if (l == 0) good = good && mbar_wait(smem_u32(&bars.g_ready), it & 1u, abort_flag);
-                            else if (ac >= 0) good = good && mbar_wait(smem_u32(&bars.a_ready[ac]), (l - 1) & 1u, abort_flag);
-                            good = good && mbar_wait(smem_u32(&bars.acc_empty[i & 1u]), ((i >> 1) & 1u) ^ 1u, abort_flag);
+                            if (l == 0) good = good && mbar_wait(smem_u32(&bars.g_ready), it & 1u, abort_flag, p.wait_ns);
+                            else if (ac >= 0) good = good && mbar_wait(smem_u32(&bars.a_ready[ac]), (l - 1) & 1u, abort_flag, p.wait_ns);
+                            good = good && mbar_wait(smem_u32(&bars.acc_empty[i & 1u]), ((i >> 1) & 1u) ^ 1u, abort_flag, p.wait_ns);
                             const uint32_t st = (2 * i + 1) % kStages, ph = ((2 * i + 1) / kStages) & 1u;
                             const bool both = mbar_try_wait(smem_u32(&bars.full[st]), ph) && mbar_try_wait(smem_u32(&bars.pfull[st]), ph);
                             const int k = !good ? 0 : (__all_sync(0xffffffffu, both) ? 2 : 1);
@@ -397,7 +399,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             // next unit, once the skip layer's MMAs have read the current one's
             uint32_t it = 0;
             for (int u = u0 + du; u < n_units && ok; u += du, ++it) {
-                if (!mbar_wait_sleep(smem_u32(&bars.g_free), it & 1u, abort_flag)) { ok = false; break; }
+                if (!mbar_wait_sleep(smem_u32(&bars.g_free), it & 1u, abort_flag, p.wait_ns)) { ok = false; break; }
     #pragma unroll 1
                 for (int q = 0; q < 4; ++q) encode(u, (it + 1) & 1u, 32 * q + lane);
             }
@@ -416,7 +418,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         float2 s[64];   // sums of the thread's 128 columns (32 of each 64)
 
         auto acquire = [&]() -> bool {
-            const bool g = mbar_wait(smem_u32(&bars.acc_full[i & 1u]), (i >> 1) & 1u, abort_flag);
+            const bool g = mbar_wait(smem_u32(&bars.acc_full[i & 1u]), (i >> 1) & 1u, abort_flag, p.wait_ns);
             tc_fence_after();
             return g;
         };
@@ -448,7 +450,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             // (written over for unit it + 2 only after the skip layer's MMAs of
             // unit it + 1, whose operands every warp here has stored after its
             // last use of unit it's)
-            if (!mbar_wait(smem_u32(&bars.ex_ready), it & 1u, abort_flag)) { ok = false; break; }
+            if (!mbar_wait(smem_u32(&bars.ex_ready), it & 1u, abort_flag, p.wait_ns)) { ok = false; break; }
             for (int l = 0; l < 8 && ok; ++l) {
                 const int nch = chunks_of(l);
 #pragma unroll
@@ -489,7 +491,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                 sm.ex_m[j][r] = (uint8_t)(__float_as_uint(m) >> 23);
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&bars.pair[quad]));
-                if (!mbar_wait(smem_u32(&bars.pair[quad]), l & 1u, abort_flag)) { ok = false; break; }
+                if (!mbar_wait(smem_u32(&bars.pair[quad]), l & 1u, abort_flag, p.wait_ns)) { ok = false; break; }
                 const uint32_t E = max(max((uint32_t)sm.ex_m[0][r], (uint32_t)sm.ex_m[1][r]), 27u);
                 const float sc = __uint_as_float((268u - E) << 23);   // 2^(14 - e)
                 const float2 sc2 = make_float2(sc, sc);
@@ -569,7 +571,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                 *scr = make_float4(o[0], o[1], o[2], sig);
                 mbar_arrive(hb);
             } else {
-                if (!mbar_wait(hb, it & 1u, abort_flag)) { ok = false; break; }
+                if (!mbar_wait(hb, it & 1u, abort_flag, p.wait_ns)) { ok = false; break; }
                 const float4 v = *scr;
                 if (valid) {
                     float4 res;
@@ -746,6 +748,8 @@ cudaError_t mlp_fp32(mcl_map* m, const Ray* rays, const float* z, int S, int n_r
     p.out = out;
     p.abort_flag = st->abort_flag;
     p.status_code = &m->status->code;
+    p.wait_ns = kWaitNs;
+    p.hold_weights = mlp_tc_take_hold(m, &p.wait_ns);
     cudaError_t e = cudaMemsetAsync(st->abort_flag, 0, sizeof(int), s);
     if (e) return e;
     const long long units = (p.M + 255) / 256;

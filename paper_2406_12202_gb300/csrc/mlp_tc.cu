@@ -117,9 +117,9 @@ struct Params {
     float4* out;
     int* abort_flag;        // per-launch: set on a timed-out wait
     int* status_code;       // map status word
-    unsigned long long wait_ns;  // limit of the bounded waits of k_mlp_tc
-    int hold_weights;       // failure-injection hook (k_mlp_tc): the weight
-                            // stream issues no copies, so the waits expire
+    unsigned long long wait_ns;  // limit of the bounded waits of k_mlp_tc, k_mlp_tc2
+    int hold_weights;       // failure-injection hook (the same kernels): the
+                            // weight stream issues no copies, so the waits expire
     // Fused ray epilogues (tiles hold whole rays: 128 % S == 0).
     //   fuse 0: write (sigma_raw, rgb) of every row to out;
     //   fuse 1: also the first pass of the hierarchical sampler: Eq. 1
@@ -1365,13 +1365,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads<EPIW>, 
 
     if (warp == 0) {
         // ------------------------------------------------ weight stream (both CTAs)
-        if (lane == 0) {
+        // (hold_weights: issues nothing, as in k_mlp_tc)
+        if (lane == 0 && !p.hold_weights) {
             uint32_t g = 0;
             bool ok = true;
             for (long long u = u0; u < n_units && ok; u += du) {
                 for (int b = 0; b < Fm::kBlocks; ++b, ++g) {
                     const uint32_t st = g % kStages, ph = (g / kStages) & 1u;
-                    if (!mbar_wait(smem_u32(&bars.empty[st]), ph ^ 1u, abort_flag)) {
+                    if (!mbar_wait(smem_u32(&bars.empty[st]), ph ^ 1u, abort_flag, p.wait_ns)) {
                         ok = false;
                         break;
                     }
@@ -1397,7 +1398,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads<EPIW>, 
             for (long long u = u0; u < n_units && ok; u += du)
                 for (int b = 0; b < Fm::kBlocks; ++b, ++g) {
                     const uint32_t st = g % kStages, ph = (g / kStages) & 1u;
-                    if (!mbar_wait(smem_u32(&bars.full[st]), ph, abort_flag)) {
+                    if (!mbar_wait(smem_u32(&bars.full[st]), ph, abort_flag, p.wait_ns)) {
                         ok = false;
                         break;
                     }
@@ -1524,15 +1525,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads<EPIW>, 
             uint32_t rdy_ph = 0;   // bit s: phase parity of a_ready[s]
             bool ok = true;
             auto wait_ready = [&](int s) -> bool {
-                const bool r = mbar_wait(smem_u32(&bars.a_ready[s]), (rdy_ph >> s) & 1u, abort_flag);
+                const bool r = mbar_wait(smem_u32(&bars.a_ready[s]), (rdy_ph >> s) & 1u, abort_flag, p.wait_ns);
                 rdy_ph ^= 1u << s;
                 return r;
             };
             // block gi present in both CTAs
             auto wait_block = [&](uint32_t gi) -> bool {
                 const uint32_t st = gi % kStages, ph = (gi / kStages) & 1u;
-                const bool r = mbar_wait(smem_u32(&bars.full[st]), ph, abort_flag);
-                const bool r2 = r && mbar_wait(smem_u32(&bars.pfull[st]), ph, abort_flag);
+                const bool r = mbar_wait(smem_u32(&bars.full[st]), ph, abort_flag, p.wait_ns);
+                const bool r2 = r && mbar_wait(smem_u32(&bars.pfull[st]), ph, abort_flag, p.wait_ns);
                 return r2;
             };
             auto release = [&](bool good) -> bool {
@@ -2187,8 +2188,6 @@ static_assert(kNumVariants == MCL_MLP_VARIANTS, "variant table");
 // pick on GB300 at 0.3 M and 2.5 M rows; BF16 2.02 against 2.13 ms for the
 // best single-CTA kernel, FP8 1.50 against 1.52 for its pair).
 constexpr int kDefaultVariant[3] = {-1, 13, 5};
-// The failure-injection hook's kernels (it is in the single-CTA kernel).
-constexpr int kHeldVariant[3] = {-1, 12, 5};
 // Point queries (rays of one sample, RayBias interleaved) on the defaults.
 void (*const kPointKernels[2])(Params) = {&k_mlp_tc2<false, 4, true, true>, &k_mlp_tc<true, 8, true, 0, true>};
 // The variant whose launch shape (threads, shared memory) the fused passes'
@@ -2645,13 +2644,12 @@ static cudaError_t mlp_tc_variant(mcl_map* m, int precision, int variant, const 
     p.wait_ns = kWaitNs;
     p.hold_weights = 0;
     int vsel = vi;
-    if (st->hold_launches > 0) {
-        // failure injection: the untuned single-CTA kernel with its weight
-        // stream held and a short wait limit
-        --st->hold_launches;
+    if (mlp_tc_take_hold(m, &p.wait_ns)) {
+        // failure injection: the untuned kernel of the precision (a tuned
+        // variant may lack the hook) with its weight stream held and a short
+        // wait limit
         p.hold_weights = 1;
-        p.wait_ns = st->hold_wait_ns;
-        vsel = fuse ? kFusedVariant[precision] : kHeldVariant[precision];
+        vsel = fuse ? kFusedVariant[precision] : kDefaultVariant[precision];
         p.wblocks = precision == MCL_PREC_FP8 ? st->fp8.wblocks : st->bf16.wblocks;
     }
     cudaError_t e = cudaMemsetAsync(st->abort_flag, 0, sizeof(int), s);
@@ -2660,7 +2658,7 @@ static cudaError_t mlp_tc_variant(mcl_map* m, int precision, int variant, const 
     // tiles, a single tile for the pipelined kernel, 512 rows for a CTA pair)
     const TcVariant& v = kVariants[vsel];
     void (*fn)(Params) = fuse ? kFusedKernels[precision == MCL_PREC_FP8][fuse->mode - 1]
-                         : st->ray_bias_step == 32 && !p.hold_weights ? kPointKernels[precision == MCL_PREC_FP8]
+                         : st->ray_bias_step == 32 ? kPointKernels[precision == MCL_PREC_FP8]
                                                    : v.fn;
     long long grid;
     if (v.cluster == 2) {
@@ -2777,6 +2775,14 @@ int mlp_tc_hold_weights(mcl_map* m, int n_launches, unsigned long long wait_ns) 
     st->hold_launches = n_launches;
     st->hold_wait_ns = wait_ns;
     return MCL_OK;
+}
+
+bool mlp_tc_take_hold(mcl_map* m, unsigned long long* wait_ns) {
+    TcState* st = (TcState*)m->tc_aux;
+    if (!st || st->hold_launches <= 0) return false;
+    --st->hold_launches;
+    *wait_ns = st->hold_wait_ns;
+    return true;
 }
 
 bool mlp_tc_tuned(const mcl_map* m, int precision) {
