@@ -398,7 +398,9 @@ static int render_passes(mcl_map* m, const float* d_poses, int N, const mcl_intr
                                            with_obs ? m->obs : nullptr),
                              "raygen")))
             return rc;
-        if ((rc = cuda_check(mlp_tc_ray_bias(m, m->gd, nr, nullptr, s), "per-ray bias"))) return rc;
+        if ((o->precision != MCL_PREC_FP32 || mlp_fp32_on_pairs(m)) &&
+            (rc = cuda_check(mlp_tc_ray_bias(m, m->gd, nr, nullptr, s), "per-ray bias")))
+            return rc;
     }
     // (the FP32 form: the densities of a pass that importance samples are
     // drawn from are those of the FMA chain)
@@ -552,7 +554,9 @@ extern "C" int mcl_query(mcl_map* m, const float* d_x, const float* d_dir, int n
     int rc;
     if ((rc = cuda_check(launch_query_setup(d_x, d_dir, n, m->rays, m->gd, m->zc, s), "query setup")))
         return rc;
-    if ((rc = cuda_check(mlp_tc_ray_bias(m, m->gd, n, nullptr, s, true, precision), "query ray bias"))) return rc;
+    if ((precision != MCL_PREC_FP32 || mlp_fp32_on_pairs(m)) &&
+        (rc = cuda_check(mlp_tc_ray_bias(m, m->gd, n, nullptr, s, true, precision), "query ray bias")))
+        return rc;
     if (precision == MCL_PREC_FP32)
         return cuda_check(mlp_fp32(m, m->rays, m->zc, 1, n, (float4*)d_out, s), "query mlp");
     return cuda_check(mlp_tc(m, precision, m->rays, m->gd, m->zc, 1, n, nullptr, (float4*)d_out, s),

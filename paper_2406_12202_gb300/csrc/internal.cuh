@@ -196,12 +196,14 @@ cudaError_t launch_weights(const float* e_ray, int N, int B, const mcl_opts& o, 
                            Status* status, cudaStream_t s);
 
 // mlp_split.cu: the FP32 form, (sigma_raw, rgb) for rows r = ray*S + k of the
-// pass (the rays' colour-head bias from mlp_tc_ray_bias).  rows_dev
-// (optional): device-side row count (n_rays * S is the bound).
+// pass.  rows_dev (optional): device-side row count (n_rays * S is the bound).
+// A map that it runs on operand pairs (mlp_fp32_on_pairs) takes the rays'
+// colour-head bias from mlp_tc_ray_bias; the SIMT kernels do not.
 // chain_density: the densities are those of the SIMT kernels' FMA chain.
 int mlp_split_prepare(mcl_map* m, const std::function<double(int, int, int)>& W,
                       const float* const* bias, const float* w_out, const float* b_out);
 void mlp_split_free(mcl_map* m);
+bool mlp_fp32_on_pairs(const mcl_map* m);
 cudaError_t mlp_fp32(mcl_map* m, const Ray* rays, const float* z, int S, int n_rays, float4* out,
                      cudaStream_t s, const int* rows_dev = nullptr, bool chain_density = false);
 

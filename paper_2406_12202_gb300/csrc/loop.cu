@@ -299,7 +299,8 @@ int enqueue_localize(mcl_map* m, int nq, float* P_user, int stride, const mcl_in
             L.plan, nq, Pc, stride, L.pix, K.fx, K.fy, K.cx, K.cy, np, o.near_z, o.far_z,
             prop ? 0 : o.jitter, o.seed, t, max_rays_run, m->rays, m->gd, m->zc, L.imgs, K.width,
             K.height, fused ? m->obs : nullptr);
-        if ((rc = cuda_check(mlp_tc_ray_bias(m, m->gd, max_rays_run, &L.plan->total_rays, s),
+        if ((!fp32 || mlp_fp32_on_pairs(m)) &&
+            (rc = cuda_check(mlp_tc_ray_bias(m, m->gd, max_rays_run, &L.plan->total_rays, s),
                              "loop ray bias")))
             return rc;
         if (prop) {

@@ -731,11 +731,16 @@ void mlp_split_free(mcl_map* m) {
     m->split = nullptr;
 }
 
+// (no state: a device without the tensor-core forms, see mlp_tc_prepare)
+bool mlp_fp32_on_pairs(const mcl_map* m) {
+    const SplitState* st = (const SplitState*)m->split;
+    return st && st->dense;
+}
+
 cudaError_t mlp_fp32(mcl_map* m, const Ray* rays, const float* z, int S, int n_rays, float4* out,
                      cudaStream_t s, const int* rows_dev, bool chain_density) {
     SplitState* st = (SplitState*)m->split;
-    if (!st) return cudaErrorNotSupported;
-    if (!st->dense) return mlp_fp32_simt(m, rays, z, S, n_rays, out, s, rows_dev, false);
+    if (!mlp_fp32_on_pairs(m)) return mlp_fp32_simt(m, rays, z, S, n_rays, out, s, rows_dev, false);
     SplitParams p = st->base;
     p.wblocks = st->wblocks;
     p.bias = st->bias;

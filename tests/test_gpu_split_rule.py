@@ -139,3 +139,23 @@ def test_pairs_are_no_further_from_fp64_than_the_chain(seed, decay):
     for col in (slice(0, 1), slice(1, 4)):
         assert np.sqrt((e[:, col] ** 2).mean()) <= np.sqrt((c[:, col] ** 2).mean())
         assert e[:, col].max() <= c[:, col].max()
+
+
+def test_maps_on_the_simt_kernels_launch_those_alone():
+    """Encoding, nine trunk and feature layers, two RGB layers and the density
+    head are 13 launches; a query adds its set-up, a render without importance
+    samples its rays and its composite.  The per-ray bias is the pairs'."""
+    import torch
+    M = lib()
+    blob = _twin(_dense(2))
+    x, d = _points(700, 1)
+    assert _query(M, blob, x, d)[1] == 1 + 13
+    gm = M.Map(blob, max_rays=64, max_samples=16, max_particles=8)
+    try:
+        P = torch.tensor(synth.random_particles(3, 8)[0], dtype=torch.float32, device="cuda")
+        px = torch.tensor([[1, 2], [9, 4], [3, 15]], dtype=torch.int32, device="cuda")
+        before = gm.profile_read()[1]
+        gm.render(P, M.intrinsics(30.0, 30.0, 8.0, 8.0, 16, 16), 2, px, M.UpdateOptions(n_coarse=16, n_fine=0))
+        assert gm.profile_read()[1] - before == 2 + 13
+    finally:
+        gm.close()
