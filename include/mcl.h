@@ -18,11 +18,11 @@
  *   weights) are recorded in a per-map status word (mcl_read_status).
  * - The library allocates device memory only in mcl_init_map (weights and a
  *   workspace sized by mcl_map_config) and frees it in mcl_destroy_map; the
- *   training and gradient entry points (mcl_proposal_train,
- *   mcl_proposal_loss_grad, mcl_fit_map, mcl_map_loss_grad) also allocate
- *   their scratch.  Up to 1 GiB of it stays with the map for the next such
- *   call, until mcl_destroy_map; a larger scratch is freed before the call
- *   returns.
+ *   training entry points (mcl_proposal_train, mcl_fit_map) also allocate
+ *   their scratch and free it before they return.  The gradient entry points
+ *   (mcl_proposal_loss_grad, mcl_map_loss_grad), made to be called step by
+ *   step, leave up to 1 GiB of theirs with the map for the next such call,
+ *   until mcl_destroy_map; a larger scratch is freed before the call returns.
  * - Every floating-point array is row-major and tightly packed.
  * - A map may be used by one stream at a time (the workspace is shared).
  */
@@ -362,7 +362,7 @@ int mcl_proposal_loss_grad(mcl_map* map, const float* d_o, const float* d_d,
  * proposal weights (set them first).  d_loss_log (optional, [epochs])
  * receives the mean loss of every epoch.  Gradients are reduced in a fixed
  * order, so the same inputs give the same weights.  Synchronous; allocates
- * its training scratch (targets, one batch of activations). */
+ * and frees its training scratch (targets, one batch of activations). */
 int mcl_proposal_train(mcl_map* map, const float* d_poses, int n_poses,
                        const int32_t* d_pixels, int B, const mcl_intrinsics* K,
                        int level, const mcl_opts* sampler_opts,
@@ -393,8 +393,8 @@ typedef struct {
  * steps on shuffled batches; d_loss_log (optional, device [steps]) receives
  * each step's batch loss.  The tensor-core forms are rebuilt from the fitted
  * weights (their calibration and kernel-variant choices start afresh, and a
- * captured mcl_localize graph is dropped).  Synchronous; allocates its
- * training scratch (about 14 KB per point of a batch).  1 <= batch,
+ * captured mcl_localize graph is dropped).  Synchronous; allocates and
+ * frees its training scratch (about 14 KB per point of a batch).  1 <= batch,
  * 1 <= n, 1 <= steps. */
 int mcl_fit_map(mcl_map* map, const float* d_x, const float* d_dir, const float* d_target, int n,
                 const mcl_fit_cfg* cfg, float* d_loss_log, void* stream);

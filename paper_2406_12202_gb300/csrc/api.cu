@@ -35,25 +35,36 @@ static std::atomic<long long> g_launches{0};
 
 void note_launch(int n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 
-int Scratch::take(mcl_map* m) {
+static void give_back(mcl_map* m) {
+    if (m->scratch) cudaFree(m->scratch);
+    m->scratch = nullptr;
+    m->scratch_bytes = 0;
+}
+
+int Scratch::take(mcl_map* m, bool keep) {
     size_t total = 0;
     for (const Piece& q : pieces_) total += (q.bytes + 255) & ~(size_t)255;
-    m_ = m;
-    char* base;
-    if (total <= kScratchKeep) {
-        if (m->scratch_bytes < total) {
-            if (m->scratch) cudaFree(m->scratch);
-            m->scratch = nullptr;
-            m->scratch_bytes = 0;
-            const int rc = cuda_check(cudaMalloc(&m->scratch, total), "scratch");
-            if (rc) return rc;
-            m->scratch_bytes = total;
+    char* base = (char*)m->scratch;
+    if (m->scratch_bytes < total) {
+        keep = keep && total <= kScratchKeep;
+        if (keep) give_back(m);
+        void* block = nullptr;
+        cudaError_t e = cudaMalloc(&block, total);
+        if (e == cudaErrorMemoryAllocation && m->scratch) {
+            // the block kept for later calls is not worth this one
+            cudaGetLastError();
+            give_back(m);
+            e = cudaMalloc(&block, total);
         }
-        base = (char*)m->scratch;
-    } else {
-        const int rc = cuda_check(cudaMalloc(&own_, total), "scratch");
+        const int rc = cuda_check(e, "scratch");
         if (rc) return rc;
-        base = (char*)own_;
+        if (keep) {
+            m->scratch = block;
+            m->scratch_bytes = total;
+        } else {
+            own_ = block;
+        }
+        base = (char*)block;
     }
     for (const Piece& q : pieces_) {
         *q.p = base;

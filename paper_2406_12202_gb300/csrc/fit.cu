@@ -70,7 +70,7 @@ int alloc_buf(mcl_map* m, Scratch& sc, FitBuf& b, long B, bool adam, cudaStream_
         sc.add(&b.m2, sizeof(float) * m->w32_n);
     }
     int rc;
-    if ((rc = sc.take(m))) return rc;
+    if ((rc = sc.take(m, !adam))) return rc;
     if (adam) {
         // on the run's own stream: the steps on s are not ordered after work of
         // the default stream, and the block may hold an earlier call's values

@@ -144,9 +144,11 @@ int fail(int code, const char* fmt, ...);
 void clear_error();
 int cuda_check(cudaError_t e, const char* what);
 // Scratch of one synchronous training or gradient call: one block of device
-// memory cut into pieces.  Up to kScratchKeep bytes stay with the map for its
-// next call (a map is used by one stream at a time); a larger block is freed
-// when the call returns.
+// memory cut into pieces.  The gradient calls, which a program's own training
+// loop makes again and again, leave up to kScratchKeep bytes with the map for
+// the next one (a map is used by one stream at a time).  A training run, whose
+// steps share one block, uses that block if it is large enough and otherwise
+// one of its own, freed when it returns, as is a block larger than kScratchKeep.
 constexpr size_t kScratchKeep = (size_t)1 << 30;
 class Scratch {
 public:
@@ -155,7 +157,9 @@ public:
     void add(T** p, size_t bytes) {
         pieces_.push_back({(void**)p, bytes});
     }
-    int take(mcl_map* m);     // allocates or reuses the block and sets the pieces
+    // allocates or reuses the block and sets the pieces; keep: a block up to
+    // kScratchKeep stays with the map
+    int take(mcl_map* m, bool keep);
     ~Scratch();
 
 private:
@@ -164,7 +168,6 @@ private:
         size_t bytes;
     };
     std::vector<Piece> pieces_;
-    mcl_map* m_ = nullptr;
     void* own_ = nullptr;     // a block that is not the map's
 };
 // Count of kernels launched by the library (api.cu).

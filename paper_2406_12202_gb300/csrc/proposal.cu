@@ -719,7 +719,7 @@ int proposal_loss_grad(mcl_map* m, const float* O, const float* D, int n, int nb
     PropBatch b{};
     Scratch sc;
     add_batch(sc, b, (long)n * nb);
-    int rc = sc.take(m);
+    int rc = sc.take(m, true);
     if (rc) return rc;
     rc = cuda_check(cudaMemsetAsync(d_loss, 0, sizeof(double), s), "clear loss");
     if (!rc)
@@ -756,7 +756,7 @@ int proposal_train(mcl_map* m, const float* d_poses, int n_poses, const int32_t*
     sc.add(&perm_d, sizeof(int) * n_rays);
     sc.add(&loss_acc, sizeof(double));
     add_batch(sc, b, (long)batch * nb);
-    if ((rc = sc.take(m))) return rc;
+    if ((rc = sc.take(m, false))) return rc;
     // 1) targets from the full sampler, in chunks of poses that fit the workspace
     const int chunk_poses = std::max(1, std::min(n_poses, m->cfg.max_rays / B));
     for (int p0 = 0; p0 < n_poses && !rc; p0 += chunk_poses) {
