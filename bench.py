@@ -7,7 +7,7 @@ importance samples per ray, Eq. 5 uncertainty, Eq. 6 rejection weights, FP64
 normalisation, systematic resampling, the motion model and the position
 spread of the refinement test).  The metric is ray-samples per second
 (rays x composited samples / time) with the MCL-update milliseconds.  The
-headline value is the plain FP32 form (the paper's precision); the BF16,
+headline value is the FP32 form (the paper's precision); the BF16,
 FP8 and learned-proposal + FP8 forms are reported beside it (key "forms")
 with their speed-up, their roofline and their error against the FP64
 oracle, and the equal-pose-error comparison runs on the analytic room map.
@@ -824,7 +824,7 @@ def run_ours(args):
     peaks, peak_src = load_peaks()
     rows = N * Bpx * ns
 
-    # ---- headline: the plain FP32 form (the paper's precision) ----------
+    # ---- headline: the FP32 form (the paper's precision) -----------------
     gpu_id = os.environ.get("CUDA_VISIBLE_DEVICES", str(local)).split(",")[0] or str(local)
     clocks = ClockSampler(gpu_id) if rank == 0 else None
     ms, phases, launches = timed(opts32, args.steps, args.warmup, profile=True, clocks=clocks)
@@ -880,7 +880,8 @@ def run_ours(args):
         roof = {"bound": "tensor", "achieved": flops / (mlp_ms / 1e3) / 1e12, "peak": peak,
                 "unit": "TFLOP/s", "peak_source": f"bf16_tflops burst ({peak_src})"
                 + (" x 2 nominal fp8/bf16 ratio" if prec == "fp8" else ""),
-                "kernel": "k_mlp_tc (coarse + fine passes)", "mlp_ms_per_step": mlp_ms}
+                "kernel": ("k_mlp_tc2 (CTA pairs" if prec == "bf16" else "k_mlp_tc (one CTA")
+                + ", the untuned kernel; coarse + fine passes)", "mlp_ms_per_step": mlp_ms}
         roof["frac"] = roof["achieved"] / roof["peak"]
         roof["achieved_survey_flops"] = 2.0 * MAC_PER_SAMPLE_FP32 * rows / (mlp_ms / 1e3) / 1e12
         roof["traffic"] = profiled_traffic(f"k_mlp_tc_c2_{prec}",
@@ -987,7 +988,8 @@ def run_ours(args):
         "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
         "config": {"workload": wl["workload"], "particles": N, "pixels": Bpx,
                    "image": f"{W}x{H}", "samples_per_ray": f"{wl['n_coarse']}+{wl['n_fine']}",
-                   "mlp_precision": "fp32 (plain form, the paper's precision)",
+                   "mlp_precision": "fp32 (the paper's precision; FP16 operand pairs with FP32 sums "
+                                    "on the tensor cores, first-pass densities on FP32 FMAs)",
                    "l2": "flushed (256 MB write) between timed steps",
                    "step": "update + resample + predict + position spread",
                    "parallelism": f"replicas x{world} (one query per GPU)"},

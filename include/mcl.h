@@ -73,6 +73,17 @@ typedef struct {
     int width, height;
 } mcl_intrinsics;
 
+/* Arithmetic of the NeRF MLP.  FP32: FP32 weights, activations and sums.  Maps
+ * whose every row of weights is a sum of many terms (He-normal ones, maps fitted
+ * from them) take their products on the tensor cores, each operand held as two
+ * FP16 numbers of 22 to 23 significant bits together, and 64 products at a time
+ * in the tensor core's accumulator, which truncates, corrected for the mean of
+ * that.  Measured against FP64, relative to the error of a chain of FP32 FMAs:
+ * densities 0.5 to 0.9 and colours 0.5 on He-normal and smooth maps, densities
+ * 1.2 to 1.4 (the largest error 0.7 to 0.8) and colours 0.4 on fitted ones.  All
+ * other maps, and the densities that importance samples are drawn from, are
+ * computed by chains of FP32 FMAs.  BF16 / FP8: operands of 8 / 4 significant
+ * bits, FP32 sums. */
 enum { MCL_PREC_FP32 = 0, MCL_PREC_BF16 = 1, MCL_PREC_FP8 = 2 };
 
 /* Options of one weight update. */
@@ -297,11 +308,10 @@ typedef struct {
  * stay on the device: with use_graph != 0 the run is captured into a CUDA
  * graph on the map's own stream (ordered after earlier work on `stream` and
  * before later work on it) and kept; later calls with the same shapes and
- * pointers relaunch it.  opts->precision selects the NeRF MLP's form (the
- * plain FP32 form or a tensor-core form); opts->use_proposal selects the
- * learned sampler.  The map must hold the largest iteration: n_queries * max(max_q
- * h_n0[q] * n_pixels[0], max_s min(n_cap[s], stride) * n_pixels[s]) <=
- * max_rays, and n_queries * stride <= max_particles. */
+ * pointers relaunch it.  opts->precision selects the NeRF MLP's form (FP32,
+ * BF16 or FP8); opts->use_proposal selects the learned sampler.  The map must
+ * hold the largest iteration: n_queries * max(max_q h_n0[q] * n_pixels[0],
+ * max_s min(n_cap[s], stride) * n_pixels[s]) <= max_rays, and n_queries * stride <= max_particles. */
 int mcl_localize(mcl_map* map, int n_queries, float* d_particles, int stride,
                  const int* h_n0, const float* const* h_images,
                  const mcl_intrinsics* K, const mcl_schedule* sch,
@@ -376,9 +386,8 @@ int mcl_proposal_train(mcl_map* map, const float* d_poses, int n_poses,
  * [n,3] (normalised here) and targets d_target [n,4] = (density, r, g, b) --
  * by minimising the mean of
  *   sigma_weight (sigma_raw(x) - density)^2 + |rgb(x, d) - (r, g, b)|^2
- * with the library's own FP32 forward (the plain form's kernels, every
- * layer's output kept), backward (SGEMMs on transposed weights with the
- * ReLU masks) and Adam.  Weight gradients are summed over each batch in a
+ * with the library's own FP32 forward (chains of FP32 FMAs, every layer's
+ * output kept), backward (the same with the ReLU masks) and Adam.  Weight gradients are summed over each batch in a
  * fixed order, so the same inputs give the same weights. */
 typedef struct {
     int steps;            /* Adam steps                                      */

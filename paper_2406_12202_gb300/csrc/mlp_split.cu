@@ -17,8 +17,11 @@
 // activations) and 2.0e-7 (all terms of one sign), against 2.0e-7 and 2.2e-7
 // of an FP32 FMA chain; emptied every 128 products 2.0e-7 and 4.9e-7, not at
 // all 3.4e-7 and 1.2e-6.  What is left is mostly a shortfall of every chunk
-// (kUnbias).  The whole MLP on six dense maps: relative error 3.1e-7 to
-// 7.1e-7, against 4.1e-7 to 1.3e-6 of the SIMT kernels (mlp_fp32.cu).
+// (kUnbias).  The whole MLP on twelve dense maps (He-normal, and smooth ones whose
+// weights fall as 2^-k with the frequency), 40,000 points each: the error of the
+// densities is 0.50 to 0.88 of the SIMT kernels' (mlp_fp32.cu), of the colours
+// 0.44 to 0.54 (rms; the largest errors 0.50 to 0.77 and 0.32 to 0.55).  Other maps
+// run on those kernels (pairs_are_exact).
 //
 // A CTA pair (the two SMs of a TPC, tcgen05 cta_group::2) walks over units of
 // 256 rows (samples of the pass, row = ray * S + k), 128 rows per CTA, through
@@ -765,8 +768,8 @@ cudaError_t mlp_fp32(mcl_map* m, const Ray* rays, const float* z, int S, int n_r
     // the FMA chain.  The inverse CDF divides its rounding (6e-8) by the
     // probability of the bin (1e-5 at least), so a density rounded otherwise,
     // even if closer to the exact one, moves samples of nearly empty bins by
-    // up to 1e-3 of a bin, and the colour of a ray in some 100,000 with them.
-    // With these densities the samples stay where they were.
+    // up to 1e-3 of a bin, and with them the colour of a ray in some 100,000, by
+    // up to 4e-3.  With these densities the samples stay where they were.
     return mlp_fp32_simt(m, rays, z, S, n_rays, out, s, rows_dev, true);
 }
 

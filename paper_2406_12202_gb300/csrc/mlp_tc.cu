@@ -2549,7 +2549,7 @@ cudaError_t mlp_tc_ray_bias(mcl_map* m, const float* gd, int n_rays, const int* 
     // Interleaved, but too few rays for a block per 32 on every SM: a warp per
     // ray all the same (scattered stores, but eight times the warps: 100 FP8 points
     // 42.6 -> 41.0 us, 1,000 BF16 points 52.9 -> 50.8; at 20,000 the block wins)
-    if (points && n_rays >= 152 * 32)
+    if (points && n_rays >= st->n_sm * 32)
         k_ray_bias<true, true><<<(unsigned)(((long)n_rays + 31) / 32), 256, 0, s>>>(gd, n_rays, n_rays_dev, st->Wd, st->bprime, out);
     else if (points)
         k_ray_bias<true, false><<<by_ray, 256, 0, s>>>(gd, n_rays, n_rays_dev, st->Wd, st->bprime, out);

@@ -194,8 +194,13 @@ __device__ __forceinline__ void importance_warp(const Ray* __restrict__ rays,
         const float sg = fmaxf(cdf[k * 33], 0.0f);
         const float delta = (zs[(k + 1) * 33] - zs[k * 33]) * dn;
         const float a = 1.0f - expf(-sg * delta);
-        // (rounded twice in every fourth bin: the samples drawn from the CDF are
-        // ill-conditioned, so its roundings are part of the result)
+        // T a + 1e-5, rounded twice in every fourth bin and once in the others.
+        // No formula asks for that: a loop unrolled by four, a thread per ray,
+        // was once compiled so, and every result since has these roundings.  The
+        // inverse CDF is ill-conditioned (an ulp here moves samples of nearly
+        // empty bins, and the weights of a few particles beyond FP32's own
+        // error), so one form for all bins would be another sampler, not a
+        // more exact one.
         const float w = (k & 3) == 3 ? __fadd_rn(__fmul_rn(T, a), 1e-5f) : fmaf(T, a, 1e-5f);
         T *= (1.0f - a);
         if (k >= 1) {
